@@ -6,11 +6,22 @@
 // Kernel structure (one CTA per SM, persistent over output tiles x K splits):
 //   warp 0     TMA producer: A tile (BM x 64, K-major, 128B swizzle) and B tile
 //              (64 x BN, N-major, 128B swizzle, 64-column boxes) into an
-//              mbarrier-guarded ring of STAGES shared-memory stages of one K
-//              block, or two for 128x64, 128x128 and the 256x128 pair.
-//   warp 1     allocates TMEM; one thread issues tcgen05.mma (M = 128, N = BN,
+//              mbarrier-guarded ring of STAGES shared-memory stages, one K block each.
+//   warp 1     allocates TMEM; one lane issues tcgen05.mma (M = 128, N = BN,
 //              K = 16) into a TMEM accumulator, double-buffered when it fits,
 //              and commits stage releases / accumulator-full to mbarriers.
+//   Both warps step through their loops converged: all lanes test the barriers, a
+//   vote makes the outcome uniform, and the loads, MMAs and commits are predicated
+//   instructions of one elected lane.  tcgen05.mma and the TMA instructions take
+//   their operands from uniform registers; in code that one lane runs by itself
+//   every operand is first moved there, which made each MMA cost about 95 cycles of
+//   issue whatever its size (N = 64 at M = 128 needs 48, bound by its operand reads;
+//   N = 128 needs 64, N = 256 needs 128).  K blocks of 64, cycles each at 2.07 GHz,
+//   512 x 512 x 4096, before and after: 128x64 390 -> 205, 128x128 385 -> 275,
+//   256x64 (two MMAs per K step) 680 -> 395, the 256x128 pair 420 -> 275,
+//   128x192 510 -> 405; 128x256 and the 256x256 tiles were at the MMA rate.
+//   Those tiles no longer gain from two K blocks in a stage (one barrier round for
+//   both): 128x64 is 8 % faster with eight stages of one, 128x128 4 % with six.
 //   warps 2-5  epilogue: tcgen05.ld of their 32 TMEM lanes, 128B-swizzled
 //              staging, TMA store (beta = 0) or TMA reduce-add (beta = 1).
 // Padding is never materialised: tensor maps carry the logical extents, so
@@ -106,18 +117,12 @@ struct GemmArgs {
 // columns of B in its shared memory, M = 256 per MMA instruction).
 template <int BM, int BN, int STAGES, int CTAS = 1>
 struct KCfg {
-  // K blocks per ring stage.  Every stage costs one full/empty barrier round, and a stage
-  // of one 64-deep K block of a 128-row tile with N <= 128 holds less MMA work than that
-  // round takes; those tiles (128x64, 128x128 and the 256x128 pair's CTAs) put two K
-  // blocks in a stage, with half as many stages in the same bytes.
-  static constexpr int SUB = (BM == 128 && BN <= 128) ? 2 : 1;
   static constexpr int A_BYTES = BM * kBK * 2;
   // B columns a CTA loads: its BN / CTAS rounded up to whole 64-column (128-byte) boxes
   // (a 256x192 pair's CTA loads 128 columns, of which its MMAs read 96)
   static constexpr int BN_LOAD = (BN / CTAS + 63) / 64 * 64;
   static constexpr int B_BYTES = kBK * BN_LOAD * 2;
-  static constexpr int SUB_BYTES = A_BYTES + B_BYTES;  // one K block: A, then B
-  static constexpr int STAGE_BYTES = SUB * SUB_BYTES;
+  static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;  // one K block: A, then B
   static constexpr int HALVES = BM / 128;
   static constexpr int ACC_COLS = HALVES * BN;
   static constexpr int NBUF = (2 * ACC_COLS <= 512) ? 2 : 1;
@@ -664,7 +669,7 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
   Unit first{};
   if constexpr (!Sched::kMapsInGlobal) {
     sched.init();
-    if (warp == 0 && lane == 0 && sched.count() > 0) first = sched.unit(0);
+    if (warp == 0 && sched.count() > 0) first = sched.unit(0);
   }
   if (!early) grid_dependency_wait();
   grid_launch_dependents();
@@ -678,59 +683,43 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
   }
 
   if (warp == 0) {
-    // ------------------------------------------------ TMA producer (one thread)
-    if (lane == 0) {
-      int stage = 0, fills = 0;
-      uint32_t ph = 0;
-      uint32_t issued_mask = 0, issued_ph = 0;
-      bool ok = true;
-      for (int i = 0; ok && i < nunits; ++i) {
-        const Unit w = (!Sched::kMapsInGlobal && i == 0) ? first : sched.unit(i);
-        if constexpr (Sched::kMapsInGlobal) {
-          tensormap_fence_acquire(w.a);
-          tensormap_fence_acquire(w.b);
+    // ------------------------------------------------ TMA producer (one elected lane issues)
+    int stage = 0, fills = 0;
+    uint32_t ph = 0;
+    uint32_t issued_mask = 0, issued_ph = 0;
+    bool ok = true;
+    const uint32_t lead = elect_one() ? 1u : 0u;
+    for (int i = 0; ok && i < nunits; ++i) {
+      const Unit w = (!Sched::kMapsInGlobal && i == 0) ? first : sched.unit(i);
+      if constexpr (Sched::kMapsInGlobal) {
+        tensormap_fence_acquire(w.a);
+        tensormap_fence_acquire(w.b);
+      }
+      for (int kb = w.kb0; kb < w.kb1; ++kb) {
+        // a stage's first fill needs no wait: nothing has used it yet
+        if (fills >= STAGES && !mbar_wait_warp(empty_bar(stage), ph ^ 1u, timeout, abort_flag)) {
+          ok = false;
+          break;
         }
-        for (int kbs = w.kb0; kbs < w.kb1; kbs += C::SUB) {
-          const int nsub = w.kb1 - kbs < C::SUB ? w.kb1 - kbs : C::SUB;  // K blocks in this stage
-          // a stage's first fill needs no wait: nothing has used it yet
-          if (fills >= STAGES && !mbar_wait(empty_bar(stage), ph ^ 1u, timeout, abort_flag)) {
-            ok = false;
-            break;
-          }
-          ++fills;
-          if constexpr (P2) {
-            // Both CTAs' loads complete on the even CTA's full barrier, which expects both halves.
-            if (sched.rank == 0) mbar_arrive_expect_tx(full_bar(stage), 2 * nsub * C::SUB_BYTES);
-            const uint32_t fb = mapa_shared(full_bar(stage), 0);
-            for (int u = 0; u < nsub; ++u) {
-              const int kb = kbs + u;
-              const uint32_t sa = sbase + stage * C::STAGE_BYTES + u * C::SUB_BYTES;
-              const uint32_t sb = sa + C::A_BYTES;
-              tma_load_2d_pair(sa, w.a, fb, kb * kBK, w.tm * BM);
+        ++fills;
+        const uint32_t sa = sbase + static_cast<uint32_t>(stage) * C::STAGE_BYTES;
+        // pair: both CTAs' loads complete on the even CTA's full barrier, which expects both halves
+        const uint32_t fb = P2 ? mapa_shared(full_bar(stage), 0) : full_bar(stage);
+        const int bx = w.tn * BN + (P2 ? sched.rank * (BN / 2) : 0);
+        mbar_arrive_expect_tx_lead(full_bar(stage), (P2 ? 2 : 1) * C::STAGE_BYTES, P2 && sched.rank != 0 ? 0u : lead);
+        tma_load_2d_lead<P2 ? 2 : 1>(sa, w.a, fb, kb * kBK, w.tm * BM, lead);
 #pragma unroll
-              for (int j = 0; j < C::BN_LOAD / 64; ++j)
-                tma_load_2d_pair(sb + j * (kBK * 128), w.b, fb, w.tn * BN + sched.rank * (BN / 2) + j * 64, kb * kBK);
-            }
-          } else {
-            mbar_arrive_expect_tx(full_bar(stage), nsub * C::SUB_BYTES);
-            for (int u = 0; u < nsub; ++u) {
-              const int kb = kbs + u;
-              const uint32_t sa = sbase + stage * C::STAGE_BYTES + u * C::SUB_BYTES;
-              const uint32_t sb = sa + C::A_BYTES;
-              tma_load_2d(sa, w.a, full_bar(stage), kb * kBK, w.tm * BM);
-#pragma unroll
-              for (int j = 0; j < BN / 64; ++j)
-                tma_load_2d(sb + j * (kBK * 128), w.b, full_bar(stage), w.tn * BN + j * 64, kb * kBK);
-            }
-          }
-          issued_mask |= 1u << stage;
-          issued_ph = (issued_ph & ~(1u << stage)) | (ph << stage);
-          if (++stage == STAGES) {
-            stage = 0;
-            ph ^= 1u;
-          }
+        for (int j = 0; j < C::BN_LOAD / 64; ++j)
+          tma_load_2d_lead<P2 ? 2 : 1>(sa + C::A_BYTES + j * (kBK * 128), w.b, fb, bx + j * 64, kb * kBK, lead);
+        issued_mask |= 1u << stage;
+        issued_ph = (issued_ph & ~(1u << stage)) | (ph << stage);
+        if (++stage == STAGES) {
+          stage = 0;
+          ph ^= 1u;
         }
       }
+    }
+    if (lane == 0) {
       if (!ok) {
         atomicExch(err, kErrProducer);
         *abort_flag = 1;
@@ -747,89 +736,77 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
         }
       }
     }
+    __syncwarp();
   } else if (warp == 1) {
-    // ------------------------------------------------ MMA issuer (one thread)
-    // Lane 0 alone runs the loop: tcgen05.mma and tcgen05.commit are issued by a
-    // single thread, and keeping the other 31 lanes out of the loop saves a warp
-    // vote and a warp reconvergence per stage (about 200 of the 550 cycles a stage
-    // cost when the whole warp stepped through it).
-    if (lane == 0) {
-      int stage = 0, acc = 0;
-      uint32_t ph = 0, aph = 0;
-      bool ok = true;
-      if (stall) ok = mbar_wait(drain_bar, 0, timeout, abort_flag);
-      // a pair's odd CTA issues nothing: the even CTA's MMAs read and write both
-      const int issue_units = (!P2 || sched.rank == 0) ? nunits : 0;
-      for (int i = 0; ok && i < issue_units; ++i) {
-        const Unit w = sched.unit(i);
-        const int kb0 = w.kb0, kb1 = w.kb1;
-        ok = mbar_wait(tempty_bar(acc), aph ^ 1u, timeout, abort_flag);
+    // ------------------------------------------------ MMA issuer (one elected lane issues)
+    int stage = 0, acc = 0;
+    uint32_t ph = 0, aph = 0;
+    bool ok = true;
+    const uint32_t lead = elect_one() ? 1u : 0u;
+    const uint64_t adesc0 = smem_desc_sw128(sbase, 16, 1024);
+    const uint64_t bdesc0 = smem_desc_sw128(sbase + C::A_BYTES, kBK * 128, 1024);
+    const uint32_t alo0 = static_cast<uint32_t>(adesc0), blo0 = static_cast<uint32_t>(bdesc0);
+    const uint32_t desc_hi = static_cast<uint32_t>(adesc0 >> 32);  // that of both: same stride and swizzle
+    if (stall) ok = mbar_wait_warp(drain_bar, 0, timeout, abort_flag);
+    // a pair's odd CTA issues nothing: the even CTA's MMAs read and write both
+    const int issue_units = (!P2 || sched.rank == 0) ? nunits : 0;
+    for (int i = 0; ok && i < issue_units; ++i) {
+      const Unit w = sched.unit(i);
+      const int kb0 = w.kb0, kb1 = w.kb1;
+      ok = mbar_wait_warp(tempty_bar(acc), aph ^ 1u, timeout, abort_flag);
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t d0 = tmem_base + static_cast<uint32_t>(acc * C::ACC_COLS);
+      for (int kb = kb0; kb < kb1; ++kb) {
+        ok = mbar_wait_warp(full_bar(stage), ph, timeout, abort_flag);
         if (!ok) break;
+        if (i == 0 && kb == kb0 && lane == 0) RG_STAMP(4);
         tc_fence_after();
-        const uint32_t d0 = tmem_base + static_cast<uint32_t>(acc * C::ACC_COLS);
-        for (int kbs = kb0; kbs < kb1; kbs += C::SUB) {
-          const int nsub = kb1 - kbs < C::SUB ? kb1 - kbs : C::SUB;  // K blocks in this stage
-          ok = mbar_wait(full_bar(stage), ph, timeout, abort_flag);
-          if (!ok) break;
-          if (i == 0 && kbs == kb0) RG_STAMP(4);
-          tc_fence_after();
-          if constexpr (Sched::kMemOnly) {
-            mbar_arrive(empty_bar(stage));  // no MMA reads the stage: it is free once its bytes have landed
-          } else {
-            for (int u = 0; u < nsub; ++u) {
-              const uint32_t sa = sbase + stage * C::STAGE_BYTES + u * C::SUB_BYTES;
-              const uint32_t sb = sa + C::A_BYTES;
-              // The descriptors of the block's K steps differ only in their start
-              // address field (bits 0-13, address >> 4; no carry: shared addresses
-              // stay below 2^18), so they are the block's base descriptors plus constants.
-              const uint64_t adesc0 = smem_desc_sw128(sa, 16, 1024);
-              const uint64_t bdesc0 = smem_desc_sw128(sb, kBK * 128, 1024);
-              const uint32_t first = kbs + u > kb0 ? 1u : 0u;
+        if constexpr (Sched::kMemOnly) {
+          if (lane == 0) mbar_arrive(empty_bar(stage));  // no MMA reads the stage: it is free once its bytes have landed
+        } else {
+          // The descriptors of the stages and K steps differ only in their start address
+          // field (bits 0-13, address >> 4; no carry: shared addresses stay below 2^18):
+          // the low words are the first stage's plus offsets, the high words constant.
+          const uint32_t so = static_cast<uint32_t>(stage) * (C::STAGE_BYTES >> 4);
+          const uint32_t first = kb > kb0 ? 1u : 0u;
 #pragma unroll
-              for (int k = 0; k < kBK / 16; ++k) {
-                const uint64_t bdesc = bdesc0 + static_cast<uint64_t>((k * 2048) >> 4);
+          for (int k = 0; k < kBK / 16; ++k) {
 #pragma unroll
-                for (int h = 0; h < C::HALVES; ++h) {
-                  const uint64_t adesc = adesc0 + static_cast<uint64_t>((h * (128 * 128) + k * 32) >> 4);
-                  if constexpr (P2)
-                    mma_f16_pair(d0, adesc, bdesc, C::IDESC, k > 0 ? 1u : first);
-                  else
-                    mma_f16(d0 + h * BN, adesc, bdesc, C::IDESC, k > 0 ? 1u : first);
-                }
-              }
-            }
-            if constexpr (P2)
-              mma_commit_pair_multicast(empty_bar(stage), 3);  // the stage is free in both CTAs
-            else
-              mma_commit(empty_bar(stage));
+            for (int h = 0; h < C::HALVES; ++h)
+              mma_f16_lead<P2 ? 2 : 1>(d0 + h * BN, alo0 + so + ((h * (128 * 128) + k * 32) >> 4), desc_hi,
+                                       blo0 + so + ((k * 2048) >> 4), desc_hi, C::IDESC, k > 0 ? 1u : first, lead);
           }
-          if (++stage == STAGES) {
-            stage = 0;
-            ph ^= 1u;
-          }
+          mma_commit_lead<P2 ? 2 : 1>(empty_bar(stage), lead);  // the stage is free (pair: in both CTAs)
         }
-        if (!ok) break;
-        if constexpr (Sched::kMemOnly)
-          mbar_arrive(tfull_bar(acc));
-        else if constexpr (P2)
-          mma_commit_pair_multicast(tfull_bar(acc), 3);  // both CTAs' halves of the accumulator are final
-        else
-          mma_commit(tfull_bar(acc));
-        if (++acc == C::NBUF) {
-          acc = 0;
-          aph ^= 1u;
+        if (++stage == STAGES) {
+          stage = 0;
+          ph ^= 1u;
         }
-        if (i + 1 == issue_units) RG_STAMP(5);
       }
-      if (!ok) {
+      if (!ok) break;
+      if constexpr (Sched::kMemOnly) {
+        if (lane == 0) mbar_arrive(tfull_bar(acc));
+      } else {
+        mma_commit_lead<P2 ? 2 : 1>(tfull_bar(acc), lead);  // pair: both CTAs' halves of the accumulator are final
+      }
+      if (++acc == C::NBUF) {
+        acc = 0;
+        aph ^= 1u;
+      }
+      if (i + 1 == issue_units && lane == 0) RG_STAMP(5);
+    }
+    if (!ok) {
+      if (elect_one()) {
         atomicExch(err, kErrMma);
         *abort_flag = 1;
         if constexpr (P2)
           mma_commit_pair(drain_bar);
         else
           mma_commit(drain_bar);  // completes once every issued MMA has finished
-        mbar_wait(drain_bar, 0, kDrainCycles, no_abort);
       }
+      __syncwarp();
+      mbar_wait_warp(drain_bar, 0, kDrainCycles, no_abort);
     }
     __syncwarp();
   } else {
@@ -1283,10 +1260,9 @@ struct TileKernel {
   int ring;             // bytes of the operand ring (the cluster split-K receive space)
 };
 
-// Stages of the cta_group::2 instances, per CTA: 16 KB of A + BN/2 x 64 of B per K block;
-// the 256x128 pair's stages hold two K blocks.
+// Stages of the cta_group::2 instances, per CTA: 16 KB of A + BN/2 x 64 of B per K block.
 template <int BN>
-constexpr int kStages2Sm = BN == 128 ? 4 : 6;
+constexpr int kStages2Sm = BN == 128 ? 8 : 6;
 
 template <int BM, int BN, int ST>
 TileKernel make_tile_kernel() {
@@ -1305,7 +1281,7 @@ TileKernel make_tile_kernel() {
 
 static const TileKernel& tile_kernel(int tile) {
   static const TileKernel table[RG_NUM_TILES] = {
-      make_tile_kernel<128, 64, 4>(),  make_tile_kernel<128, 128, 3>(), make_tile_kernel<128, 256, 4>(),
+      make_tile_kernel<128, 64, 8>(),  make_tile_kernel<128, 128, 6>(), make_tile_kernel<128, 256, 4>(),
       make_tile_kernel<256, 64, 4>(),  make_tile_kernel<256, 128, 4>(), make_tile_kernel<256, 256, 3>(),
       make_tile_kernel<128, 192, 4>(), make_tile_kernel<256, 192, 3>(),
   };
@@ -1319,7 +1295,7 @@ using GroupedFn = void (*)(const GroupHeader*, const GroupItem*, const CUtensorM
                            long long);
 static const void* grouped_kernel(int family) {
   static const GroupedFn table[kGroupFamilies] = {
-      gemm_bf16_grouped_kernel<128, 64, 4>,  gemm_bf16_grouped_kernel<128, 128, 3>,
+      gemm_bf16_grouped_kernel<128, 64, 8>,  gemm_bf16_grouped_kernel<128, 128, 6>,
       gemm_bf16_grouped_kernel<128, 256, 4>, gemm_bf16_grouped_kernel<256, 64, 4>,
       gemm_bf16_grouped_kernel<256, 128, 4>, gemm_bf16_grouped_kernel<256, 256, 3>,
       gemm_bf16_grouped_kernel<128, 192, 4>, gemm_bf16_grouped_kernel<256, 192, 3>,
