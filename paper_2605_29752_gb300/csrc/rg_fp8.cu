@@ -10,19 +10,29 @@
 // units; BN = 256 or 128; split S = 1, 2, 4 or 8):
 //   warp 0     TMA producer: A block 128 x 128 bytes (K-major) and B block 128 K-rows
 //              x BN bytes (N-major, 128-byte-wide column boxes), 128-byte swizzle.
-//   warp 1     one thread issues tcgen05.mma kind::f8f6f4 (M = 128, N = BN, K = 32) into
-//              one of 512 / BN TMEM buffers, a fresh accumulator per 128-deep K block,
-//              and commits once per K block to the buffer's full barrier.
+//   warp 1     one lane issues tcgen05.mma kind::f8f6f4 (M = 128, K = 32) into a fresh TMEM
+//              accumulator per 128-deep K block (128 x 256: one per 128-column half), and commits
+//              each to its buffer's full barrier.  Warps 0 and 1 step converged with predicated
+//              loads, MMAs and commits, as in the BF16 kernels, and for the same reason: with one
+//              lane in the loop by itself a K block took its thread 750 cycles (128 x 128) to 1000
+//              (128 x 256) for 256 and 512 cycles of MMAs.
 //   warps 2-3  idle: they complete warpgroup 0, whose registers go to the promotion warps.
 //   warps 4-11 promotion and epilogue (224 registers each), two warps per TMEM lane
 //              quarter, each owning one half of the tile's columns: per K block, tcgen05.ld
-//              the block product 64 columns per wait, multiply by sA * sB (one scalar per
-//              warp and K block) and add into FP32 registers; after the unit's last block,
-//              128B-swizzled staging and a TMA store (beta = 0) or reduce-add (beta = 1).
+//              the block product in 32-column chunks, the next on its way while one is added,
+//              multiply by sA * sB (one scalar per warp and K block) and add into FP32 registers;
+//              the buffer is released once its last chunk has arrived.  After the unit's last
+//              block, 128B-swizzled staging and a TMA store (beta = 0) or reduce-add (beta = 1).
 //              With S > 1 the unit's partial goes to the split-K workspace instead, and the
 //              last arriving split of a (tile, warp) sums the S partials in the fixed order
-//              0..S-1.  Their release of a buffer (and, through warp 4, of the K block's
-//              operand stage) is what lets the producer and the MMA thread reuse it.
+//              0..S-1.  Their release of a buffer (and of the K block's operand stage) is what
+//              lets the producer and the MMA warp reuse it.
+// What bounds it: at 512 x 1536 x 2048 (48 CTAs of 128 x 128) about 360 cycles per K block against
+// 256 of MMAs, the buffer's round trip through the promotion; on 128 x 256 about 700 against 512,
+// where the MMAs alone take 620 and the promotion alone 580.  Before and after these three changes
+// (converged issue, chunked promotion, halves), sweep protocol: 512 x 1536 x 2048 on 128 x 128 9.2 ->
+// 7.1 us; 3072 x 2048 x 4096 38.3 -> 27.1 (128 x 128), 37.6 -> 30.4 (128 x 256); 4096^3 73.8 -> 60.8
+// (128 x 256), 73.2 -> 62.2 (the pair); 8192^2 x 4096 251 -> 209 and 247 -> 210.
 // The 256 x 256 tile also runs as a tcgen05 cta_group::2 pair (gemm_fp8_2sm_kernel):
 // each CTA of a 2-CTA cluster loads its 128 rows of A and 128 columns of B, the even
 // CTA issues the M = 256 MMAs, and each CTA promotes and stores its own 128 rows.
@@ -62,7 +72,6 @@ static_assert(4 * kRegsLow + kEpiWarps * kRegsHigh == (kThreads / 32) * kLaunchR
 static_assert(kRegsLow + 2 * kRegsHigh == 3 * kLaunchRegs, "register split per sub-partition");
 constexpr int BM = 128, BK = 128;             // BK: one 128-byte swizzle row of e4m3 = one scale block
 constexpr int SB = 128;                       // scale block edge
-constexpr int STAGING_PER_WARP = 2 * 4096;
 constexpr long long kDrainCycles = 1LL << 30;
 constexpr uint32_t FULL = 0xffffffffu;
 
@@ -71,23 +80,31 @@ constexpr uint32_t FULL = 0xffffffffu;
 template <int BN, bool PAIR = false>
 struct Cfg {
   static constexpr int CTAS = PAIR ? 2 : 1;
-  static constexpr int STAGES = PAIR ? 5 : BN == 256 ? 3 : 4;
+  // Column halves of a K block, an MMA and a TMEM accumulator buffer each: the 1-CTA 128x256
+  // tile alone has two, so that a buffer comes back after half a K block's promotion.  It then
+  // takes four operand stages (TMA latency, not the MMAs, bound it with three: 4096^3 63.2 us
+  // against 60.8) for one staging buffer per promotion warp instead of two.  In the pair the
+  // halves' MMAs (64 of each CTA's 128 columns) were slower: 62.2 against 66.5 us.
+  static constexpr int HALVES = BN == 256 && !PAIR ? 2 : 1;
+  static constexpr int STAGES = PAIR ? 5 : 4;
+  static constexpr int NSTG = HALVES == 2 ? 1 : 2;  // staging buffers per promotion warp
   static constexpr int A_BYTES = BM * BK;
   static constexpr int B_BYTES = BK * BN / CTAS;  // (BN / CTAS) / 128 N-major column boxes of BK rows
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int NACC = 512 / BN;       // TMEM accumulator buffers of BN columns: all 512 columns
-  static constexpr int TMEM_COLS = NACC * BN;
+  static constexpr int NB = BN / HALVES;      // columns of an MMA and of a TMEM accumulator buffer
+  static constexpr int DEPTH = 512 / BN;      // K blocks in flight in TMEM (all 512 columns)
+  static constexpr int NACC = DEPTH * HALVES; // accumulator buffers
   static constexpr int STAGING_OFF = STAGES * STAGE_BYTES;
-  static constexpr int BAR_OFF = STAGING_OFF + kEpiWarps * STAGING_PER_WARP;
+  static constexpr int BAR_OFF = STAGING_OFF + kEpiWarps * NSTG * 4096;
   static constexpr int SMEM_BYTES = 1024 + BAR_OFF + 256;
   static constexpr int HALF = BN / 2;         // columns per promotion warp
-  static constexpr int LDG = 64;              // columns of a K block's product read per TMEM wait
   // E4M3 x E4M3, A K-major, B MN-major; M = 256 across a pair
-  static constexpr uint32_t IDESC = instr_desc(0, 0, 0, 1, 128 * CTAS, BN);
+  static constexpr uint32_t IDESC = instr_desc(0, 0, 0, 1, 128 * CTAS, NB);
   static_assert(SMEM_BYTES <= 232448, "shared memory budget");
   static_assert(BN == 128 || BN == 256, "tile width");
   static_assert(!PAIR || BN == 256, "pair tile");
   static_assert((2 * STAGES + 2 * NACC + 1) * 8 + 8 <= 256, "barrier block");
+  static_assert(STAGES * STAGE_BYTES % 1024 == 0, "staging alignment");
 };
 
 template <uint32_t N>
@@ -106,15 +123,21 @@ __device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t cluster_add
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 
-// D (+)= A * B across a CTA pair (cta_group::2, M = 256 per instruction), e4m3 inputs, F32 accumulator.
-__device__ __forceinline__ void mma_f8_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                            uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
+// a0 = sc * p0 + a0, a1 = sc * p1 + a1, each rounded once: two FMAs, or one two-wide FMA (the same
+// results), which saves issue slots and pays where a warp holds 128 accumulators (pair, 4096^3: 64.2
+// against 62.2 us) and not where it holds 64 (128x128 at 8192^2 x 4096: 262 against 267 us).
+template <bool WIDE>
+__device__ __forceinline__ void add_scaled(float& a0, float& a1, uint32_t p0, uint32_t p1, float sc) {
+  if constexpr (WIDE) {
+    asm("{\n\t.reg .b64 x, y, z;\n\t"
+        "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %4};\n\tmov.b64 z, {%0, %1};\n\t"
+        "fma.rn.f32x2 z, x, y, z;\n\tmov.b64 {%0, %1}, z;\n\t}"
+        : "+f"(a0), "+f"(a1)
+        : "r"(p0), "r"(p1), "f"(sc));
+  } else {
+    a0 = fmaf(sc, __uint_as_float(p0), a0);
+    a1 = fmaf(sc, __uint_as_float(p1), a1);
+  }
 }
 
 struct Args {
@@ -139,9 +162,10 @@ __device__ __forceinline__ void st_shared_v4(uint32_t addr, float a, float b, fl
 
 // One warp writes a 32 x 32 FP32 block (lane = row) through swizzled staging
 // with a TMA store, or a TMA reduce-add when add is set.
+template <int NSTG>
 __device__ __forceinline__ void put_block(const CUtensorMap* map, const float* v, int row0, int col0, bool add,
                                           uint32_t stg0, int& sbuf, int lane) {
-  if (lane == 0) bulk_wait_read<1>();
+  if (lane == 0) bulk_wait_read<NSTG - 1>();
   __syncwarp();
   const uint32_t buf = stg0 + sbuf * 4096;
 #pragma unroll
@@ -156,7 +180,7 @@ __device__ __forceinline__ void put_block(const CUtensorMap* map, const float* v
       tma_store_2d(map, buf, col0, row0);
     bulk_commit();
   }
-  sbuf ^= 1;
+  if constexpr (NSTG > 1) sbuf ^= 1;
 }
 
 // The kernel body.  SPLIT = false: the instance for S = 1 (no workspace path, so its
@@ -169,16 +193,13 @@ template <int BN, bool SPLIT, bool PAIR>
 __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmC,
                                          const CUtensorMap& tmW, const Args& args) {
   using C = Cfg<BN, PAIR>;
-  // Coupled ring (as many stages as accumulator buffers, one CTA: the 128x128 tile): K block kb
-  // uses stage kb % STAGES and buffer kb % NACC, the same index.  The producer refills a stage
-  // only once the promotion warps have released its buffer, which they do after the block's
-  // MMAs completed, so a landed stage also means a free buffer: the MMA thread waits on one
-  // barrier and commits to one per K block.
-  constexpr bool COUPLED = C::NACC == C::STAGES && !PAIR;
-  // Otherwise the MMA thread commits only to the accumulator-full barrier, and the first
-  // promotion warp of each CTA frees the K block's stage once it has seen that barrier (the
-  // block's MMAs, which read the stage, have completed): one commit per K block, not two.
-  constexpr bool STAGE_BY_PROMOTION = !COUPLED;
+  // Coupled ring (as many stages as K blocks in TMEM, one CTA: the 128x128 tile): K block kb
+  // uses stage and buffer kb % STAGES.  The producer refills a stage only once the promotion
+  // warps have released its buffer, which they do after the block's MMAs completed, so a landed
+  // stage also means a free buffer and the MMA warp waits on one barrier per K block.
+  constexpr bool COUPLED = C::DEPTH == C::STAGES && !PAIR;
+  // Otherwise the first promotion warp of the last half frees the K block's stage once it has
+  // seen that half's products (every MMA that reads the stage has then completed).
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_s = smem_u32(smem_raw);
   uint8_t* smem = smem_raw + ((1024u - (raw_s & 1023u)) & 1023u);
@@ -228,7 +249,8 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
     }
     for (int b = 0; b < C::NACC; ++b) {
       mbar_init(tfull_bar(b), 1);
-      mbar_init(tempty_bar(b), PAIR ? 2 * kEpiWarps : kEpiWarps);  // pair: both CTAs' warps, on the even CTA
+      // released by the warps that promote it (pair: both CTAs', on the even CTA)
+      mbar_init(tempty_bar(b), C::CTAS * kEpiWarps / C::HALVES);
     }
     mbar_init(drain_bar, 1);
     *abort_flag = 0;
@@ -236,10 +258,10 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
   }
   if (warp == 1) {
     if constexpr (PAIR) {  // collective with the partner's warp 1: the same columns in both CTAs
-      tmem_alloc_pair(smem_u32(tmem_slot), C::TMEM_COLS);
+      tmem_alloc_pair(smem_u32(tmem_slot), 512);
       tmem_relinquish_pair();
     } else {
-      tmem_alloc(smem_u32(tmem_slot), C::TMEM_COLS);
+      tmem_alloc(smem_u32(tmem_slot), 512);
       tmem_relinquish();
     }
   }
@@ -255,44 +277,40 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
   if (warp < kEpiWarp0) {
     setmaxnreg_dec<kRegsLow>();
     if (warp == 0) {
-      if (lane == 0) {
-        int stage = 0, fills = 0;
-        uint32_t ph = 0, issued_mask = 0, issued_ph = 0;
-        bool ok = true;
-        for (int u = cid; ok && u < total; u += ncl) {
-          const int s = u % S;
-          int tm, tn;
-          tile_of(u, tm, tn);
-          const int kb1 = s + 1 == S ? args.kblocks : kb_lo(s + 1);
-          for (int kb = kb_lo(s); kb < kb1; ++kb) {
-            if (fills >= C::STAGES &&
-                !mbar_wait(COUPLED ? tempty_bar(stage) : empty_bar(stage), ph ^ 1u, args.timeout, abort_flag)) {
-              ok = false;
-              break;
-            }
-            ++fills;
-            const uint32_t sa = sbase + stage * C::STAGE_BYTES;
-            if constexpr (PAIR) {
-              // both CTAs' loads complete on the even CTA's full barrier, which expects both halves
-              if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), 2 * C::STAGE_BYTES);
-              const uint32_t fb = mapa_shared(full_bar(stage), 0);
-              tma_load_2d_pair(sa, &tmA, fb, kb * BK, tm * BM);
-              tma_load_2d_pair(sa + C::A_BYTES, &tmB, fb, tn * BN + rank * (BN / 2), kb * BK);
-            } else {
-              mbar_arrive_expect_tx(full_bar(stage), C::STAGE_BYTES);
-              tma_load_2d(sa, &tmA, full_bar(stage), kb * BK, tm * BM);
+      int stage = 0, fills = 0;
+      uint32_t ph = 0, issued_mask = 0, issued_ph = 0;
+      bool ok = true;
+      const uint32_t lead = elect_one() ? 1u : 0u;
+      for (int u = cid; ok && u < total; u += ncl) {
+        const int s = u % S;
+        int tm, tn;
+        tile_of(u, tm, tn);
+        const int kb1 = s + 1 == S ? args.kblocks : kb_lo(s + 1);
+        for (int kb = kb_lo(s); kb < kb1; ++kb) {
+          if (fills >= C::STAGES &&
+              !mbar_wait_warp(COUPLED ? tempty_bar(stage) : empty_bar(stage), ph ^ 1u, args.timeout, abort_flag)) {
+            ok = false;
+            break;
+          }
+          ++fills;
+          const uint32_t sa = sbase + static_cast<uint32_t>(stage) * C::STAGE_BYTES;
+          // pair: both CTAs' loads complete on the even CTA's full barrier, which expects both halves
+          const uint32_t fb = PAIR ? mapa_shared(full_bar(stage), 0) : full_bar(stage);
+          const int bx = tn * BN + (PAIR ? rank * (BN / 2) : 0);
+          mbar_arrive_expect_tx_lead(full_bar(stage), C::CTAS * C::STAGE_BYTES, PAIR && rank != 0 ? 0u : lead);
+          tma_load_2d_lead<C::CTAS>(sa, &tmA, fb, kb * BK, tm * BM, lead);
 #pragma unroll
-              for (int j = 0; j < BN / 128; ++j)
-                tma_load_2d(sa + C::A_BYTES + j * (BK * 128), &tmB, full_bar(stage), tn * BN + j * 128, kb * BK);
-            }
-            issued_mask |= 1u << stage;
-            issued_ph = (issued_ph & ~(1u << stage)) | (ph << stage);
-            if (++stage == C::STAGES) {
-              stage = 0;
-              ph ^= 1u;
-            }
+          for (int j = 0; j < BN / C::CTAS / 128; ++j)
+            tma_load_2d_lead<C::CTAS>(sa + C::A_BYTES + j * (BK * 128), &tmB, fb, bx + j * 128, kb * BK, lead);
+          issued_mask |= 1u << stage;
+          issued_ph = (issued_ph & ~(1u << stage)) | (ph << stage);
+          if (++stage == C::STAGES) {
+            stage = 0;
+            ph ^= 1u;
           }
         }
+      }
+      if (lane == 0) {
         if (!ok) {
           atomicExch(args.err, 1);
           *abort_flag = 1;
@@ -309,64 +327,64 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
           }
         }
       }
+      __syncwarp();
     } else if (warp == 1) {
-      // Lane 0 alone issues the MMAs and commits (no per-K-block warp vote); a pair's
-      // odd CTA issues nothing: the even CTA's MMAs read and write both.
-      if (lane == 0 && (!PAIR || rank == 0)) {
+      // A pair's odd CTA issues nothing: the even CTA's MMAs read and write both.
+      if (!PAIR || rank == 0) {
         int stage = 0, acc = 0;
         uint32_t ph = 0, aph = 0;
         bool ok = true;
+        const uint32_t lead = elect_one() ? 1u : 0u;
+        // descriptors of stage 0: the stages and K steps differ in the start address field of the low words
+        const uint64_t adesc0 = smem_desc_sw128(sbase, 16, 1024);
+        const uint64_t bdesc0 = smem_desc_sw128(sbase + C::A_BYTES, BK * 128, 1024);  // column boxes BK*128 apart
+        const uint32_t alo0 = static_cast<uint32_t>(adesc0), blo0 = static_cast<uint32_t>(bdesc0);
+        const uint32_t desc_hi = static_cast<uint32_t>(adesc0 >> 32);  // that of both: same stride and swizzle
         for (int u = cid; ok && u < total; u += ncl) {
           const int s = u % S;
           const int kb1 = s + 1 == S ? args.kblocks : kb_lo(s + 1);
           for (int kb = kb_lo(s); kb < kb1; ++kb) {
-            if constexpr (!COUPLED) {
-              ok = mbar_wait(tempty_bar(acc), aph ^ 1u, args.timeout, abort_flag);
-              if (!ok) break;
-            }
-            ok = mbar_wait(full_bar(stage), ph, args.timeout, abort_flag);
+            ok = mbar_wait_warp(full_bar(stage), ph, args.timeout, abort_flag);
             if (!ok) break;
-            tc_fence_after();
-            const uint32_t sa = sbase + stage * C::STAGE_BYTES;
-            const uint32_t sb = sa + C::A_BYTES;
-            const uint32_t d = tmem_base + static_cast<uint32_t>(acc * BN);
-            // K steps differ only in the descriptors' start address field (address >> 4)
-            const uint64_t adesc0 = smem_desc_sw128(sa, 16, 1024);
-            const uint64_t bdesc0 = smem_desc_sw128(sb, BK * 128, 1024);  // column boxes BK*128 apart
+            const uint32_t so = static_cast<uint32_t>(stage) * (C::STAGE_BYTES >> 4);
 #pragma unroll
-            for (int k = 0; k < BK / 32; ++k) {
-              const uint64_t ad = adesc0 + static_cast<uint64_t>((k * 32) >> 4);
-              const uint64_t bd = bdesc0 + static_cast<uint64_t>((k * (32 * 128)) >> 4);
-              if constexpr (PAIR)
-                mma_f8_pair(d, ad, bd, C::IDESC, k > 0 ? 1u : 0u);
-              else
-                mma_f8(d, ad, bd, C::IDESC, k > 0 ? 1u : 0u);
+            for (int h = 0; h < C::HALVES; ++h) {
+              const int buf = acc * C::HALVES + h;
+              if constexpr (!COUPLED) {
+                if (ok) ok = mbar_wait_warp(tempty_bar(buf), aph ^ 1u, args.timeout, abort_flag);
+                if (!ok) break;
+              }
+              tc_fence_after();
+              constexpr uint32_t hb = (BK * 128) >> 4;  // half h of the B columns is the h-th column box
+#pragma unroll
+              for (int k = 0; k < BK / 32; ++k)
+                mma_f8_lead<C::CTAS>(tmem_base + static_cast<uint32_t>(buf * C::NB), alo0 + so + ((k * 32) >> 4), desc_hi,
+                                     blo0 + so + h * hb + ((k * (32 * 128)) >> 4), desc_hi, C::IDESC, k > 0 ? 1u : 0u,
+                                     lead);
+              mma_commit_lead<C::CTAS>(tfull_bar(buf), lead);  // pair: both CTAs' rows of the product are ready
             }
-            if constexpr (PAIR) {
-              if constexpr (!STAGE_BY_PROMOTION) mma_commit_pair_multicast(empty_bar(stage), 3);
-              mma_commit_pair_multicast(tfull_bar(acc), 3);    // both CTAs' rows of the product are ready
-            } else {
-              if constexpr (!COUPLED && !STAGE_BY_PROMOTION) mma_commit(empty_bar(stage));
-              mma_commit(tfull_bar(acc));
-            }
+            if (!ok) break;
             if (++stage == C::STAGES) {
               stage = 0;
               ph ^= 1u;
             }
-            if (++acc == C::NACC) {
+            if (++acc == C::DEPTH) {
               acc = 0;
               aph ^= 1u;
             }
           }
         }
         if (!ok) {
-          atomicExch(args.err, 2);
-          *abort_flag = 1;
-          if constexpr (PAIR)
-            mma_commit_pair(drain_bar);
-          else
-            mma_commit(drain_bar);  // completes once every issued MMA has finished
-          mbar_wait(drain_bar, 0, kDrainCycles, no_abort);
+          if (elect_one()) {
+            atomicExch(args.err, 2);
+            *abort_flag = 1;
+            if constexpr (PAIR)
+              mma_commit_pair(drain_bar);
+            else
+              mma_commit(drain_bar);  // completes once every issued MMA has finished
+          }
+          __syncwarp();
+          mbar_wait_warp(drain_bar, 0, kDrainCycles, no_abort);
         }
       }
       __syncwarp();
@@ -377,7 +395,7 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
     const int e = warp - kEpiWarp0;
     const int q = warp & 3;
     const int hc = e / 4;
-    const uint32_t stg0 = sbase + C::STAGING_OFF + e * STAGING_PER_WARP;
+    const uint32_t stg0 = sbase + C::STAGING_OFF + e * (C::NSTG * 4096);
     int acc = 0, sbuf = 0, pstage = 0;  // pstage: the operand stage of the current K block
     uint32_t aph = 0;
     bool ok = true;
@@ -406,38 +424,40 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
                                          : 0.f;
         }
         const float sc = __shfl_sync(FULL, sc_lane, rel & 31);
-        ok = __all_sync(FULL, mbar_wait(tfull_bar(acc), aph, args.timeout, abort_flag));
+        const int buf = C::HALVES == 2 ? 2 * acc + hc : acc;
+        ok = mbar_wait_warp(tfull_bar(buf), aph, args.timeout, abort_flag);
         if (!ok) break;
-        if constexpr (STAGE_BY_PROMOTION) {
-          if (e == 0 && lane == 0) mbar_arrive(empty_bar(pstage));  // this CTA's copy of the stage is free
+        if constexpr (!COUPLED) {
+          if (e == (C::HALVES - 1) * 4 && lane == 0) mbar_arrive(empty_bar(pstage));  // this CTA's copy of the stage is free
           if (++pstage == C::STAGES) pstage = 0;
         }
         tc_fence_after();
         const uint32_t t = tmem_base + (static_cast<uint32_t>(q * 32) << 16) +
-                           static_cast<uint32_t>(acc * BN + hc * C::HALF);
+                           static_cast<uint32_t>(buf * C::NB + (C::HALVES == 2 ? 0 : hc * C::HALF));
+        // 32 columns at a time: the next 32 are on their way while these are added, and the
+        // buffer is released as soon as the last have arrived, before they are added.
+        uint32_t p[2][32];
+        tmem_ld_32x32b_x32(t, p[0]);
+        tmem_ld_wait_for(p[0]);
 #pragma unroll
-        for (int c = 0; c < C::HALF / C::LDG; ++c) {
-          uint32_t p[C::LDG / 32][32];
-#pragma unroll
-          for (int j = 0; j < C::LDG / 32; ++j) tmem_ld_32x32b_x32(t + c * C::LDG + j * 32, p[j]);
-          tmem_ld_wait();
-#pragma unroll
-          for (int j = 0; j < C::LDG / 32; ++j)
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-              float& acc_v = r[c * C::LDG + j * 32 + i];
-              acc_v = fmaf(sc, __uint_as_float(p[j][i]), acc_v);
+        for (int c = 0; c < C::HALF / 32; ++c) {
+          if (c + 1 < C::HALF / 32) {
+            tmem_ld_32x32b_x32(t + (c + 1) * 32, p[(c + 1) & 1]);
+          } else {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) {
+              if constexpr (PAIR)
+                mbar_arrive_cluster_relaxed(mapa_shared(tempty_bar(buf), 0));  // the even CTA's MMA reuses it
+              else
+                mbar_arrive(tempty_bar(buf));
             }
+          }
+#pragma unroll
+          for (int i = 0; i < 32; i += 2) add_scaled<BN == 256>(r[c * 32 + i], r[c * 32 + i + 1], p[c & 1][i], p[c & 1][i + 1], sc);
+          if (c + 1 < C::HALF / 32) tmem_ld_wait_for(p[(c + 1) & 1]);
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) {
-          if constexpr (PAIR)
-            mbar_arrive_cluster_relaxed(mapa_shared(tempty_bar(acc), 0));  // the even CTA's MMA reuses it
-          else
-            mbar_arrive(tempty_bar(acc));
-        }
-        if (++acc == C::NACC) {
+        if (++acc == C::DEPTH) {
           acc = 0;
           aph ^= 1u;
         }
@@ -448,7 +468,7 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
 #pragma unroll
         for (int c = 0; c < C::HALF / 32; ++c) {
           const int col0 = tn * BN + hc * C::HALF + c * 32;
-          if (row0 < args.M && col0 < args.N) put_block(&tmC, r + c * 32, row0, col0, args.beta != 0, stg0, sbuf, lane);
+          if (row0 < args.M && col0 < args.N) put_block<C::NSTG>(&tmC, r + c * 32, row0, col0, args.beta != 0, stg0, sbuf, lane);
         }
         continue;
       }
@@ -457,12 +477,12 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
       const bool direct = !SPLIT || S == 1;
       const CUtensorMap* dst = direct ? &tmC : &tmW;
       const int drow = direct ? row0 : (s * ntiles + tile) * BM + q * 32;
-      const int dcol = direct ? tn * BN + hc * C::HALF : hc * C::HALF;
+      const int dcol = direct ? tn * BN : 0;
       const bool dadd = direct && args.beta != 0;
 #pragma unroll
       for (int c = 0; c < C::HALF / 32; ++c)
-        if (!direct || (row0 < args.M && dcol + c * 32 < args.N))
-          put_block(dst, r + c * 32, drow, dcol + c * 32, dadd, stg0, sbuf, lane);
+        if (!direct || (row0 < args.M && dcol + hc * C::HALF + c * 32 < args.N))
+          put_block<C::NSTG>(dst, r + c * 32, drow, dcol + hc * C::HALF + c * 32, dadd, stg0, sbuf, lane);
       if (direct) continue;
       if constexpr (SPLIT) {
       // Split-K: wait for this split's stores, fence them against the generic
@@ -507,7 +527,7 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
           }
         }
         const int col0 = tn * BN + hc * C::HALF + c * 32;
-        if (row0 < args.M && col0 < args.N) put_block(&tmC, sum, row0, col0, args.beta != 0, stg0, sbuf, lane);
+        if (row0 < args.M && col0 < args.N) put_block<C::NSTG>(&tmC, sum, row0, col0, args.beta != 0, stg0, sbuf, lane);
       }
       }
     }
@@ -527,9 +547,9 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
   if (warp == 1) {
     tc_fence_after();
     if constexpr (PAIR)
-      tmem_dealloc_pair(tmem_base, C::TMEM_COLS);
+      tmem_dealloc_pair(tmem_base, 512);
     else
-      tmem_dealloc(tmem_base, C::TMEM_COLS);
+      tmem_dealloc(tmem_base, 512);
   }
 }
 
