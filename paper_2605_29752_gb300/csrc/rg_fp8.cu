@@ -572,29 +572,64 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 
 // One CTA per 128 x 128 block: amax, scale = amax / 448 (1 for an all-zero
 // block), codes = e4m3(x / scale) rounded to nearest even with saturation.
-__global__ void __launch_bounds__(256) quantize_kernel(const float* __restrict__ X, int64_t rows, int64_t cols,
-                                                       int64_t ldx, uint8_t* __restrict__ Q, int64_t ldq,
-                                                       float* __restrict__ scales, int64_t s_ld) {
-  __shared__ float red[8];
-  const int64_t r0 = static_cast<int64_t>(blockIdx.y) * 128, c0 = static_cast<int64_t>(blockIdx.x) * 128;
-  const int tid = threadIdx.x;
+// Bound by HBM (5 bytes per element).  X is read once, its block held in registers
+// between the amax and the codes (eight rows per warp, four columns per lane), with
+// 16-byte loads and 4-byte stores of four codes where VEC (X 16-byte aligned, ldx a
+// multiple of 4, Q 4-byte aligned, ldq a multiple of 4); else, and at a ragged right
+// edge, element by element.
+constexpr int kQThreads = 512, kQRows = 128 / (kQThreads / 32);  // rows per warp
+template <bool VEC>
+__global__ void __launch_bounds__(kQThreads, 2) quantize_kernel(const float* __restrict__ X, int64_t rows, int64_t cols,
+                                                                int64_t ldx, uint8_t* __restrict__ Q, int64_t ldq,
+                                                                float* __restrict__ scales, int64_t s_ld) {
+  __shared__ float red[kQThreads / 32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t r0 = static_cast<int64_t>(blockIdx.y) * 128 + warp;  // the warp's rows: r0 + i * (warps)
+  const int64_t c = static_cast<int64_t>(blockIdx.x) * 128 + 4 * lane;
+  const bool whole = VEC && c + 4 <= cols;
+  float x[kQRows][4];
   float amax = 0.f;
-  for (int i = tid; i < 128 * 128; i += 256) {
-    const int64_t r = r0 + i / 128, c = c0 + i % 128;
-    if (r < rows && c < cols) amax = fmaxf(amax, fabsf(X[r * ldx + c]));
+#pragma unroll
+  for (int i = 0; i < kQRows; ++i) {
+    const int64_t r = r0 + i * (kQThreads / 32);
+    const float* src = X + r * ldx + c;
+    if (whole && r < rows) {
+      const float4 v = __ldcs(reinterpret_cast<const float4*>(src));
+      x[i][0] = v.x;
+      x[i][1] = v.y;
+      x[i][2] = v.z;
+      x[i][3] = v.w;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) x[i][j] = (r < rows && c + j < cols) ? src[j] : 0.f;
+    }
   }
+#pragma unroll
+  for (int i = 0; i < kQRows; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) amax = fmaxf(amax, fabsf(x[i][j]));
   for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-  if ((tid & 31) == 0) red[tid >> 5] = amax;
+  if (lane == 0) red[warp] = amax;
   __syncthreads();
   float m = red[0];
-  for (int w = 1; w < 8; ++w) m = fmaxf(m, red[w]);
+#pragma unroll
+  for (int w = 1; w < kQThreads / 32; ++w) m = fmaxf(m, red[w]);
   const float s = m > 0.f ? __fdiv_rn(m, 448.0f) : 1.0f;
-  if (tid == 0) scales[static_cast<int64_t>(blockIdx.y) * s_ld + blockIdx.x] = s;
-  for (int i = tid; i < 128 * 128; i += 256) {
-    const int64_t r = r0 + i / 128, c = c0 + i % 128;
-    if (r < rows && c < cols) {
-      const float v = __fdiv_rn(X[r * ldx + c], s);
-      Q[r * ldq + c] = static_cast<uint8_t>(__nv_cvt_float_to_fp8(v, __NV_SATFINITE, __NV_E4M3));
+  if (threadIdx.x == 0) scales[static_cast<int64_t>(blockIdx.y) * s_ld + blockIdx.x] = s;
+#pragma unroll
+  for (int i = 0; i < kQRows; ++i) {
+    const int64_t r = r0 + i * (kQThreads / 32);
+    const float2 lo = make_float2(__fdiv_rn(x[i][0], s), __fdiv_rn(x[i][1], s));
+    const float2 hi = make_float2(__fdiv_rn(x[i][2], s), __fdiv_rn(x[i][3], s));
+    const uint32_t q = static_cast<uint32_t>(__nv_cvt_float2_to_fp8x2(lo, __NV_SATFINITE, __NV_E4M3)) |
+                       static_cast<uint32_t>(__nv_cvt_float2_to_fp8x2(hi, __NV_SATFINITE, __NV_E4M3)) << 16;
+    uint8_t* dst = Q + r * ldq + c;
+    if (whole && r < rows) {
+      *reinterpret_cast<uint32_t*>(dst) = q;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (r < rows && c + j < cols) dst[j] = static_cast<uint8_t>(q >> (8 * j));
     }
   }
 }
@@ -799,8 +834,11 @@ extern "C" int rg_fp8_quantize(rg_ctx* ctx, const float* X, int64_t rows, int64_
   if (!X || !Q || !scales) return rg::fail(RG_ERR_INVALID, "rg_fp8_quantize: null pointer");
   const int64_t br = (rows + 127) / 128, bc = (cols + 127) / 128;
   if (br > 65535 || bc > (1LL << 31) - 1) return rg::fail(RG_ERR_SHAPE, "rg_fp8_quantize: too many blocks");
-  rg::fp8::quantize_kernel<<<dim3(static_cast<unsigned>(bc), static_cast<unsigned>(br)), 256, 0,
-                             static_cast<cudaStream_t>(stream)>>>(X, rows, cols, ldx, Q, ldq, scales, bc);
+  const bool vec = !(reinterpret_cast<uintptr_t>(X) & 15) && ldx % 4 == 0 && !(reinterpret_cast<uintptr_t>(Q) & 3) &&
+                   ldq % 4 == 0;
+  (vec ? rg::fp8::quantize_kernel<true> : rg::fp8::quantize_kernel<false>)<<<
+      dim3(static_cast<unsigned>(bc), static_cast<unsigned>(br)), rg::fp8::kQThreads, 0,
+      static_cast<cudaStream_t>(stream)>>>(X, rows, cols, ldx, Q, ldq, scales, bc);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? RG_OK : rg::fail(RG_ERR_CUDA, std::string("rg_fp8_quantize: ") + cudaGetErrorString(e));
 }
