@@ -570,66 +570,104 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   fp8_body<256, SPLIT, true>(tmA, tmB, tmC, tmW, args);
 }
 
+__device__ __forceinline__ uint32_t e4m3x4(float a, float b, float c, float d) {
+  return static_cast<uint32_t>(__nv_cvt_float2_to_fp8x2(make_float2(a, b), __NV_SATFINITE, __NV_E4M3)) |
+         static_cast<uint32_t>(__nv_cvt_float2_to_fp8x2(make_float2(c, d), __NV_SATFINITE, __NV_E4M3)) << 16;
+}
+
 // One CTA per 128 x 128 block: amax, scale = amax / 448 (1 for an all-zero
 // block), codes = e4m3(x / scale) rounded to nearest even with saturation.
 // Bound by HBM (5 bytes per element).  X is read once, its block held in registers
-// between the amax and the codes (eight rows per warp, four columns per lane), with
+// between the amax and the codes (a warp's rows in turn, four columns per lane), with
 // 16-byte loads and 4-byte stores of four codes where VEC (X 16-byte aligned, ldx a
 // multiple of 4, Q 4-byte aligned, ldq a multiple of 4); else, and at a ragged right
 // edge, element by element.
-constexpr int kQThreads = 512, kQRows = 128 / (kQThreads / 32);  // rows per warp
-template <bool VEC>
-__global__ void __launch_bounds__(kQThreads, 2) quantize_kernel(const float* __restrict__ X, int64_t rows, int64_t cols,
-                                                                int64_t ldx, uint8_t* __restrict__ Q, int64_t ldq,
-                                                                float* __restrict__ scales, int64_t s_ld) {
-  __shared__ float red[kQThreads / 32];
+// The codes are those of the rounded quotient x / s, found without dividing: with
+// i = 1 / s rounded, x i (1 - 2^-21) and x i (1 + 2^-21) lie below and above x / s by at
+// least 2^-22 of it (each of their three roundings moves them by at most 2^-24), so below
+// and above its rounding to FP32; e4m3 rounding is monotonic, so where both give the same
+// code it is the quotient's.  Where they differ (about one group of four in 10^4) the
+// quotients are divided.  A scale outside [2^-100, 2^100] divides everywhere (there 1 / s
+// may overflow or lose bits).
+// 4096^2: 90 us reading X twice with 4-byte accesses; 21.2 in one pass with divisions; 15.4
+// with the products, programmatic dependent launch and unguarded accesses in the interior
+// blocks (512 threads); 14.4 with 256 threads, three CTAs an SM (12.4 at the measured HBM
+// rate); 8192^2: 309 -> 50.4, 98 % of that rate.  512 threads are the faster where the blocks
+// make less than two waves of them (1024 x 4096: 4.7 against 5.5 us) and at ragged edges,
+// whose guarded blocks take longer (4000 x 4004: 18.0 against 24.2 us).
+template <bool VEC, int T>
+__global__ void __launch_bounds__(T, T == 256 ? 3 : 2)
+    quantize_kernel(const float* __restrict__ X, int64_t rows, int64_t cols, int64_t ldx, uint8_t* __restrict__ Q,
+                    int64_t ldq, float* __restrict__ scales, int64_t s_ld) {
+  constexpr int kWarps = T / 32, kRows = 128 / kWarps;  // warps, rows per warp
+  __shared__ float red[kWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t r0 = static_cast<int64_t>(blockIdx.y) * 128 + warp;  // the warp's rows: r0 + i * (warps)
+  const int64_t r0 = static_cast<int64_t>(blockIdx.y) * 128 + warp;  // the warp's rows: r0 + i * kWarps
   const int64_t c = static_cast<int64_t>(blockIdx.x) * 128 + 4 * lane;
-  const bool whole = VEC && c + 4 <= cols;
-  float x[kQRows][4];
-  float amax = 0.f;
+  const bool whole = VEC && c + 4 <= cols;  // the lane's four columns are a vector
+  // an interior block, the same for the whole CTA: its loads and stores have no guards between them
+  const bool inner = VEC && (static_cast<int64_t>(blockIdx.y) + 1) * 128 <= rows &&
+                     (static_cast<int64_t>(blockIdx.x) + 1) * 128 <= cols;
+  const float* src = X + r0 * ldx + c;
+  uint8_t* dst = Q + r0 * ldq + c;
+  grid_dependency_wait();
+  grid_launch_dependents();
+  float4 x[kRows];
+  if (inner) {
 #pragma unroll
-  for (int i = 0; i < kQRows; ++i) {
-    const int64_t r = r0 + i * (kQThreads / 32);
-    const float* src = X + r * ldx + c;
-    if (whole && r < rows) {
-      const float4 v = __ldcs(reinterpret_cast<const float4*>(src));
-      x[i][0] = v.x;
-      x[i][1] = v.y;
-      x[i][2] = v.z;
-      x[i][3] = v.w;
-    } else {
+    for (int i = 0; i < kRows; ++i) x[i] = __ldcs(reinterpret_cast<const float4*>(src + i * kWarps * ldx));
+  } else {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) x[i][j] = (r < rows && c + j < cols) ? src[j] : 0.f;
+    for (int i = 0; i < kRows; ++i) {
+      const float* p = src + i * kWarps * ldx;
+      const bool in = r0 + i * kWarps < rows;
+      if (whole && in) {
+        x[i] = __ldcs(reinterpret_cast<const float4*>(p));
+      } else {
+        x[i].x = (in && c < cols) ? p[0] : 0.f;
+        x[i].y = (in && c + 1 < cols) ? p[1] : 0.f;
+        x[i].z = (in && c + 2 < cols) ? p[2] : 0.f;
+        x[i].w = (in && c + 3 < cols) ? p[3] : 0.f;
+      }
     }
   }
+  float amax = 0.f;
 #pragma unroll
-  for (int i = 0; i < kQRows; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) amax = fmaxf(amax, fabsf(x[i][j]));
+  for (int i = 0; i < kRows; ++i)
+    amax = fmaxf(fmaxf(fmaxf(fmaxf(amax, fabsf(x[i].x)), fabsf(x[i].y)), fabsf(x[i].z)), fabsf(x[i].w));
   for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
   if (lane == 0) red[warp] = amax;
   __syncthreads();
   float m = red[0];
 #pragma unroll
-  for (int w = 1; w < kQThreads / 32; ++w) m = fmaxf(m, red[w]);
+  for (int w = 1; w < kWarps; ++w) m = fmaxf(m, red[w]);
   const float s = m > 0.f ? __fdiv_rn(m, 448.0f) : 1.0f;
   if (threadIdx.x == 0) scales[static_cast<int64_t>(blockIdx.y) * s_ld + blockIdx.x] = s;
+  const bool divide = !(s >= 0x1p-100f && s <= 0x1p100f);
+  const float inv = __fdiv_rn(1.0f, s);
+  const float lo = inv * (1.0f - 0x1p-21f), hi = inv * (1.0f + 0x1p-21f);
+  auto codes = [&](const float4& v) {
+    uint32_t q = e4m3x4(v.x * lo, v.y * lo, v.z * lo, v.w * lo);
+    if (divide || q != e4m3x4(v.x * hi, v.y * hi, v.z * hi, v.w * hi))
+      q = e4m3x4(__fdiv_rn(v.x, s), __fdiv_rn(v.y, s), __fdiv_rn(v.z, s), __fdiv_rn(v.w, s));
+    return q;
+  };
+  if (inner) {
 #pragma unroll
-  for (int i = 0; i < kQRows; ++i) {
-    const int64_t r = r0 + i * (kQThreads / 32);
-    const float2 lo = make_float2(__fdiv_rn(x[i][0], s), __fdiv_rn(x[i][1], s));
-    const float2 hi = make_float2(__fdiv_rn(x[i][2], s), __fdiv_rn(x[i][3], s));
-    const uint32_t q = static_cast<uint32_t>(__nv_cvt_float2_to_fp8x2(lo, __NV_SATFINITE, __NV_E4M3)) |
-                       static_cast<uint32_t>(__nv_cvt_float2_to_fp8x2(hi, __NV_SATFINITE, __NV_E4M3)) << 16;
-    uint8_t* dst = Q + r * ldq + c;
-    if (whole && r < rows) {
-      *reinterpret_cast<uint32_t*>(dst) = q;
-    } else {
+    for (int i = 0; i < kRows; ++i) *reinterpret_cast<uint32_t*>(dst + i * kWarps * ldq) = codes(x[i]);
+  } else {
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (r < rows && c + j < cols) dst[j] = static_cast<uint8_t>(q >> (8 * j));
+    for (int i = 0; i < kRows; ++i) {
+      const uint32_t q = codes(x[i]);
+      uint8_t* p = dst + i * kWarps * ldq;
+      const bool in = r0 + i * kWarps < rows;
+      if (whole && in) {
+        *reinterpret_cast<uint32_t*>(p) = q;
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (in && c + j < cols) p[j] = static_cast<uint8_t>(q >> (8 * j));
+      }
     }
   }
 }
@@ -836,10 +874,18 @@ extern "C" int rg_fp8_quantize(rg_ctx* ctx, const float* X, int64_t rows, int64_
   if (br > 65535 || bc > (1LL << 31) - 1) return rg::fail(RG_ERR_SHAPE, "rg_fp8_quantize: too many blocks");
   const bool vec = !(reinterpret_cast<uintptr_t>(X) & 15) && ldx % 4 == 0 && !(reinterpret_cast<uintptr_t>(Q) & 3) &&
                    ldq % 4 == 0;
-  (vec ? rg::fp8::quantize_kernel<true> : rg::fp8::quantize_kernel<false>)<<<
-      dim3(static_cast<unsigned>(bc), static_cast<unsigned>(br)), rg::fp8::kQThreads, 0,
-      static_cast<cudaStream_t>(stream)>>>(X, rows, cols, ldx, Q, ldq, scales, bc);
-  const cudaError_t e = cudaGetLastError();
+  rg::Fp8CtxInfo info{};
+  const int rc = rg::ctx_fp8_info(ctx, &info);
+  if (rc != RG_OK) return rc;
+  using rg::fp8::quantize_kernel;
+  // the 256-thread kernel: whole blocks, more than two waves of 512-thread CTAs
+  const bool many = vec && rows % 128 == 0 && cols % 128 == 0 && bc * br > 4LL * info.sms;
+  const auto fn = many ? quantize_kernel<true, 256> : vec ? quantize_kernel<true, 512> : quantize_kernel<false, 512>;
+  int64_t s_ld = bc;
+  void* params[8] = {&X, &rows, &cols, &ldx, &Q, &ldq, &scales, &s_ld};
+  const cudaError_t e = rg::fp8_launch_pdl(reinterpret_cast<const void*>(fn),
+                                           dim3(static_cast<unsigned>(bc), static_cast<unsigned>(br)), many ? 256 : 512, 0,
+                                           static_cast<cudaStream_t>(stream), params);
   return e == cudaSuccess ? RG_OK : rg::fail(RG_ERR_CUDA, std::string("rg_fp8_quantize: ") + cudaGetErrorString(e));
 }
 

@@ -47,6 +47,8 @@ def _run(rg, ctx, x, ldx, x_off, ldq, q_off):
     (64, 256, 256, 1, 256, 0),         # X one element off 16 bytes
     (64, 256, 256, 0, 256, 2),         # Q two bytes off four
     (3, 1, 1, 0, 1, 0),                # one column
+    (3200, 3200, 3204, 4, 3208, 4),    # more whole blocks than two waves of 512-thread CTAs: the 256-thread kernel
+    (3201, 3204, 3204, 0, 3204, 0),    # as many, ragged
 ])
 def test_quantizer_alignments_and_edges(rg, ctx, R, N, ldx, x_off, ldq, q_off):
     x = (synthetic.normal_stream_f32(3, 1, R * N) * np.exp2(synthetic.uniform24(3, 2, R * N) * 60 - 30)).astype(
@@ -73,3 +75,25 @@ def test_quantizer_non_finite(rg, ctx, x_off):
     assert np.isinf(s[0, 1])
     assert np.array_equal(q[:, 128:256], np.where(np.isinf(mid), 0x7F, np.where(np.signbit(mid), 0x80, 0)))
     assert s[0, 2] == 1.0 and np.all(q[:, 256:] == 0x7F)
+
+
+@pytest.mark.parametrize("exp", [0, 3, 99, 101, -99, -101, -130, -142])
+def test_quantizer_at_rounding_boundaries(rg, ctx, exp):
+    """Quotients on, and a few units in the last place around, every midpoint and value of e4m3, for scales that
+    are and are not powers of two and on both sides of the range in which no division is made."""
+    grid = np.unique(np.abs(of.e4m3_decode(np.arange(0x7F, dtype=np.uint8))))
+    marks = np.concatenate([grid, (grid[1:] + grid[:-1]) / 2])
+    blocks = []
+    for m in (1.0, 1.1, 1.7, 1.9999999):
+        amax = np.float32(np.ldexp(448.0 * m, exp))
+        s = np.float32(amax / np.float32(448.0))
+        at = (marks * np.float64(s)).astype(np.float32)
+        near = np.concatenate([at] + [at * np.float32(1 + d * 2.0 ** -23) for d in (-9, -5, -3, -1, 1, 3, 5, 9)])
+        near = np.minimum(near, amax)
+        near = np.resize(np.concatenate([near, -near]), 128 * 128)
+        near[-1] = amax
+        blocks.append(near.reshape(128, 128))
+    x = np.concatenate(blocks, axis=1)
+    q_ref, s_ref = of.quantize_blocks(x)
+    q, s = _run(rg, ctx, x, 512, 0, 512, 0)
+    assert np.array_equal(s, s_ref) and np.array_equal(q, q_ref)
