@@ -211,6 +211,10 @@ __device__ __forceinline__ void store_block(const CUtensorMap* tmC, const float 
   sbuf ^= 1;
 }
 
+// Whether a tile's grouped units may run all K splits of a problem in turn: its epilogue threads
+// then hold one FP32 sum per accumulator column (TMEM columns: BN, twice that for 256-row CTAs).
+__host__ __device__ constexpr bool serial_tile(int acc_cols) { return acc_cols <= 128; }
+
 // One work unit: which output tile of which problem, which K blocks, and where
 // its operands and output live.
 struct Unit {
@@ -226,6 +230,7 @@ struct Unit {
   int tile, ntiles;  // tile id / tile count of the problem (split-K workspace and tickets)
   int ws_row0 = 0;   // first workspace row of the problem's partials (grouped launches)
   int tk0 = 0;       // first ticket of the problem (grouped launches)
+  int segs = 1;      // > 1: this unit runs all K splits of its tile, one accumulator after another (grouped launches)
 };
 
 // Tile order: the tile grid is cut into column panels `panel` tiles wide and
@@ -506,19 +511,26 @@ struct TwoSmSched {
 // its split-K partials and tickets in the launch's workspace.  TWO_SM: units are
 // (256-row pair tile, split) and every 2-CTA cluster runs one at a time as a
 // tcgen05 cta_group::2 unit (tiles_m counts 128-row tiles).
-// Work-list records keep CUtensorMap's 128-byte alignment: a 128-byte header,
-// then 512-byte items (three maps and the sizes).
+// Work-list records keep CUtensorMap's 128-byte alignment: a 128-byte header, the
+// items' first units (4 bytes each, padded to 128 bytes), then 512-byte items (three
+// maps and the sizes).  Finding a unit's item reads the 4-byte array only, 32 entries
+// to a warp load, from the last unit's item on: a CTA's units ascend.
 struct alignas(128) GroupItem {
   CUtensorMap a, b, c;
   int32_t M, N, beta, tiles_m;
   int32_t tiles_n, kblocks, unit_start, splits;
-  int32_t ws_row0, tk0, reserved[2];
+  int32_t ws_row0, tk0;
+  int32_t segs;  // K splits one unit runs in turn (splits is then 1), or 1
+  int32_t reserved;
 };
 struct alignas(128) GroupHeader {
   int32_t n_items;
   int32_t total_units;
   int32_t reserved[30];
 };
+__host__ __device__ constexpr size_t group_items_offset(int n) {
+  return sizeof(GroupHeader) + (static_cast<size_t>(n) * 4 + 127) / 128 * 128;
+}
 
 template <bool TWO_SM>
 struct GroupSched {
@@ -527,14 +539,20 @@ struct GroupSched {
   static constexpr bool k2Sm = TWO_SM;
   static constexpr bool kSplit = true;
   const GroupHeader* h;
-  const GroupItem* items;
   const CUtensorMap* w;      // the launch's split-K workspace
   int n_items = 0, total_units = 0;  // read after the grid dependency wait
+  const int32_t* starts = nullptr;
+  const GroupItem* items = nullptr;
   int rank = 0, cid = 0, ncl = 1;
+  // the calling warp's current item and its sizes (unit() is called by whole warps, in ascending order)
+  mutable int cur = 0, loaded = -1;
+  mutable int4 d0, d1, d2;  // {M, N, beta, tiles_m}, {tiles_n, kblocks, unit_start, splits}, {ws_row0, tk0, segs, -}
   __device__ __forceinline__ void prefetch() const {}
   __device__ __forceinline__ void init() {
     n_items = h->n_items;
     total_units = h->total_units;
+    starts = reinterpret_cast<const int32_t*>(h + 1);
+    items = reinterpret_cast<const GroupItem*>(reinterpret_cast<const unsigned char*>(h) + group_items_offset(n_items));
     if constexpr (TWO_SM) {
       rank = static_cast<int>(cluster_ctarank());
       cid = static_cast<int>(blockIdx.x) / 2;
@@ -547,39 +565,68 @@ struct GroupSched {
   __device__ __forceinline__ int count() const {
     return cid < total_units ? (total_units - 1 - cid) / ncl + 1 : 0;
   }
+  // Makes the maps of this CTA's units current, by all of its threads before its warps part.
+  __device__ __forceinline__ void acquire_maps() const {
+    const int n = count();
+    for (int i = static_cast<int>(threadIdx.x); i < n; i += kThreads) {
+      const int u = cid + i * ncl;
+      int lo = 0, hi = n_items - 1;  // the last item whose first unit is <= u
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (starts[mid] <= u) lo = mid; else hi = mid - 1;
+      }
+      if (i > 0 && starts[lo] <= u - ncl) continue;  // the CTA's previous unit is of the same item
+      const GroupItem* it = items + lo;
+      tensormap_fence_acquire(&it->a);
+      tensormap_fence_acquire(&it->b);
+      tensormap_fence_acquire(&it->c);
+      prefetch_tmap(&it->a);
+      prefetch_tmap(&it->b);
+      prefetch_tmap(&it->c);
+    }
+    __syncthreads();
+  }
   __device__ __forceinline__ Unit unit(int i) const {
     const int u = cid + i * ncl;
-    int lo = 0, hi = n_items - 1;  // last item whose unit_start <= u
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (items[mid].unit_start <= u) lo = mid; else hi = mid - 1;
+    for (;;) {  // the last item whose first unit is <= u
+      const int j = cur + static_cast<int>(threadIdx.x & 31);
+      const int n = __popc(__ballot_sync(FULL, j < n_items && starts[j] <= u));  // cur itself is one
+      cur += n - 1;
+      if (n < 32) break;
     }
-    const GroupItem& it = items[lo];
+    const GroupItem* it = items + cur;
+    if (cur != loaded) {
+      const int4* f = reinterpret_cast<const int4*>(&it->M);
+      d0 = f[0];
+      d1 = f[1];
+      d2 = f[2];
+      loaded = cur;
+    }
+    const int tiles_n = d1.x, kblocks = d1.y, splits = d1.w, v = u - d1.z;
     Unit x;
     if constexpr (TWO_SM) {
-      const int v = u - it.unit_start;
-      const int p = v / it.splits;
-      x.a = &it.a;
-      x.b = &it.b;
-      x.c = &it.c;
+      const int p = v / splits;
+      x.a = &it->a;
+      x.b = &it->b;
+      x.c = &it->c;
       x.w = w;
-      x.tm = 2 * (p / it.tiles_n) + rank;  // tiles_m (128-row tiles) is even: pairs never overhang
-      x.tn = p % it.tiles_n;
-      x.s = v % it.splits;
-      x.splits = it.splits;
-      x.kb0 = it.splits == 1 ? 0 : x.s * it.kblocks / it.splits;
-      x.kb1 = it.splits == 1 ? it.kblocks : (x.s + 1) * it.kblocks / it.splits;
-      x.M = it.M;
-      x.N = it.N;
-      x.beta = it.beta;
-      x.ntiles = it.tiles_m * it.tiles_n;
-      x.tile = x.tm * it.tiles_n + x.tn;
+      x.tm = 2 * (p / tiles_n) + rank;  // tiles_m (128-row tiles) is even: pairs never overhang
+      x.tn = p % tiles_n;
+      x.s = v % splits;
+      x.splits = splits;
+      x.kb0 = splits == 1 ? 0 : x.s * kblocks / splits;
+      x.kb1 = splits == 1 ? kblocks : (x.s + 1) * kblocks / splits;
+      x.M = d0.x;
+      x.N = d0.y;
+      x.beta = d0.z;
+      x.ntiles = d0.w * tiles_n;
+      x.tile = x.tm * tiles_n + x.tn;
     } else {
-      x = split_unit(&it.a, &it.b, &it.c, w, u - it.unit_start, it.tiles_m, it.tiles_n, it.splits, it.kblocks, it.M,
-                     it.N, it.beta, it.tiles_n);
+      x = split_unit(&it->a, &it->b, &it->c, w, v, d0.w, tiles_n, splits, kblocks, d0.x, d0.y, d0.z, tiles_n);
     }
-    x.ws_row0 = it.ws_row0;
-    x.tk0 = it.tk0;
+    x.ws_row0 = d2.x;
+    x.tk0 = d2.y;
+    x.segs = d2.z;
     return x;
   }
 };
@@ -601,6 +648,8 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
   constexpr bool P2 = Sched::k2Sm;  // one CTA of a cta_group::2 pair
   constexpr bool CS = IsClusterSplit<Sched>::value;  // one K slice of a cluster split-K tile
   using C = KCfg<BM, BN, STAGES, P2 ? 2 : 1>;
+  // units may run all K splits of their tile (a thread then holds its sums of the whole tile in registers)
+  constexpr bool SERIAL = Sched::kMapsInGlobal && serial_tile(C::ACC_COLS);
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_s = smem_u32(smem_raw);
   uint8_t* smem = smem_raw + ((1024u - (raw_s & 1023u)) & 1023u);
@@ -673,7 +722,10 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
   }
   if (!early) grid_dependency_wait();
   grid_launch_dependents();
-  if constexpr (Sched::kMapsInGlobal) sched.init();
+  if constexpr (Sched::kMapsInGlobal) {
+    sched.init();
+    sched.acquire_maps();
+  }
   const int nunits = sched.count();
   if (threadIdx.x == 0) {
     RG_STAMP(3);
@@ -691,10 +743,6 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
     const uint32_t lead = elect_one() ? 1u : 0u;
     for (int i = 0; ok && i < nunits; ++i) {
       const Unit w = (!Sched::kMapsInGlobal && i == 0) ? first : sched.unit(i);
-      if constexpr (Sched::kMapsInGlobal) {
-        tensormap_fence_acquire(w.a);
-        tensormap_fence_acquire(w.b);
-      }
       for (int kb = w.kb0; kb < w.kb1; ++kb) {
         // a stage's first fill needs no wait: nothing has used it yet
         if (fills >= STAGES && !mbar_wait_warp(empty_bar(stage), ph ^ 1u, timeout, abort_flag)) {
@@ -750,9 +798,19 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
     if (stall) ok = mbar_wait_warp(drain_bar, 0, timeout, abort_flag);
     // a pair's odd CTA issues nothing: the even CTA's MMAs read and write both
     const int issue_units = (!P2 || sched.rank == 0) ? nunits : 0;
-    for (int i = 0; ok && i < issue_units; ++i) {
-      const Unit w = sched.unit(i);
-      const int kb0 = w.kb0, kb1 = w.kb1;
+    // the K range and segments of the next unit, looked up while the current one's MMAs run
+    int kb0n = 0, kb1n = 0, segsn = 1;
+    if (issue_units > 0) {
+      const Unit w = sched.unit(0);
+      kb0n = w.kb0;
+      kb1n = w.kb1;
+      segsn = w.segs;
+    }
+    int seg = 0;
+    for (int i = 0; ok && i < issue_units;) {
+      // the unit's K blocks, or those of its K split `seg`
+      const int kb0 = SERIAL && segsn > 1 ? seg * kb1n / segsn : kb0n;
+      const int kb1 = SERIAL && segsn > 1 ? (seg + 1) * kb1n / segsn : kb1n;
       ok = mbar_wait_warp(tempty_bar(acc), aph ^ 1u, timeout, abort_flag);
       if (!ok) break;
       tc_fence_after();
@@ -794,7 +852,16 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
         acc = 0;
         aph ^= 1u;
       }
-      if (i + 1 == issue_units && lane == 0) RG_STAMP(5);
+      if (SERIAL && ++seg < segsn) continue;
+      seg = 0;
+      if (++i < issue_units) {
+        const Unit w = sched.unit(i);
+        kb0n = w.kb0;
+        kb1n = w.kb1;
+        segsn = w.segs;
+      } else if (lane == 0) {
+        RG_STAMP(5);
+      }
     }
     if (!ok) {
       if (elect_one()) {
@@ -823,9 +890,6 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
     for (int i = 0; i < nunits; ++i) {
       const Unit w = sched.unit(i);
       const int tile = w.tile, s = w.s, tm = w.tm, tn = w.tn, kb0 = w.kb0, kb1 = w.kb1, ntiles = w.ntiles;
-      if constexpr (Sched::kMapsInGlobal) {
-        if (lane == 0) tensormap_fence_acquire(w.c);
-      }
       ok = __all_sync(FULL, mbar_wait(tfull_bar(acc), aph, timeout, abort_flag));
       if (!ok) break;
       if (i == 0 && warp == 2 && lane == 0) RG_STAMP(6);
@@ -900,6 +964,55 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
           }
           store_block(w.c, sum, tm * BM + (j / kCols) * 128 + q * 32, tn * BN + (j % kCols) * 32, w.M, w.N, w.beta,
                       stg0, sbuf, lane);
+        }
+      } else if (SERIAL && w.segs > 1) {
+        // All K splits of the tile, one accumulator after another: their sum in the order
+        // 0..S-1, as the workspace path's last arriver forms it, without the partials' round
+        // trip through memory (publishing, waiting for and re-reading a split's partial takes an
+        // epilogue warp 3-6 us: 8 problems of 512 x 576 x 1024 on 128x64, S = 4, 59.5 us; without
+        // a split 18.5).
+        if constexpr (SERIAL) {
+          // -0 is the sum's neutral element (-0 + x = x, also for x = -0)
+          float sum[C::ACC_COLS / 32][32];
+#pragma unroll
+          for (int c = 0; c < C::ACC_COLS / 32; ++c)
+#pragma unroll
+            for (int e = 0; e < 32; ++e) sum[c][e] = -0.f;
+#pragma unroll 1
+          for (int seg = 0; seg < w.segs; ++seg) {
+            if (seg > 0) {
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) {
+                if constexpr (P2)
+                  mbar_arrive_cluster(mapa_shared(tempty_bar(acc), 0));
+                else
+                  mbar_arrive(tempty_bar(acc));
+              }
+              if (++acc == C::NBUF) {
+                acc = 0;
+                aph ^= 1u;
+              }
+              ok = mbar_wait_warp(tfull_bar(acc), aph, timeout, abort_flag);
+              if (!ok) break;
+              tc_fence_after();
+            }
+            const bool some = (seg + 1) * kb1 / w.segs > seg * kb1 / w.segs;  // the split has K blocks
+            const uint32_t t = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * C::ACC_COLS);
+#pragma unroll
+            for (int c = 0; c < C::ACC_COLS / 32; ++c) {
+              uint32_t v[32];
+              tmem_ld_32x32b_x32(t + c * 32, v);
+              tmem_ld_wait_for(v);
+#pragma unroll
+              for (int e = 0; e < 32; ++e) sum[c][e] += some ? __uint_as_float(v[e]) : 0.f;
+            }
+          }
+          if (!ok) break;
+#pragma unroll
+          for (int c = 0; c < C::ACC_COLS / 32; ++c)
+            store_block(w.c, sum[c], tm * BM + (c * 32 / BN) * 128 + q * 32, tn * BN + c * 32 % BN, w.M, w.N, w.beta, stg0,
+                        sbuf, lane);
         }
       } else if (!Sched::kSplit || w.splits == 1) {
 #pragma unroll 1
@@ -1213,10 +1326,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 template <int BM, int BN, int STAGES>
 __global__ void __launch_bounds__(kThreads, 1)
-    gemm_bf16_grouped_kernel(const GroupHeader* __restrict__ hdr, const GroupItem* __restrict__ items,
-                             const __grid_constant__ CUtensorMap tmW, float* ws, int32_t* tickets, int32_t* err,
-                             long long timeout) {
-  GroupSched<false> sched{hdr, items, &tmW};
+    gemm_bf16_grouped_kernel(const GroupHeader* __restrict__ hdr, const __grid_constant__ CUtensorMap tmW, float* ws,
+                             int32_t* tickets, int32_t* err, long long timeout) {
+  GroupSched<false> sched{hdr, &tmW};
   gemm_body<BM, BN, STAGES>(sched, ws, tickets, err, timeout, 0, 0);
 }
 
@@ -1224,10 +1336,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 // two CTAs, so a graph kernel node launches it as pairs without a launch attribute.
 template <int BN, int STAGES>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-    gemm_bf16_grouped_2sm_kernel(const GroupHeader* __restrict__ hdr, const GroupItem* __restrict__ items,
-                                 const __grid_constant__ CUtensorMap tmW, float* ws, int32_t* tickets, int32_t* err,
-                                 long long timeout) {
-  GroupSched<true> sched{hdr, items, &tmW};
+    gemm_bf16_grouped_2sm_kernel(const GroupHeader* __restrict__ hdr, const __grid_constant__ CUtensorMap tmW,
+                                 float* ws, int32_t* tickets, int32_t* err, long long timeout) {
+  GroupSched<true> sched{hdr, &tmW};
   gemm_body<128, BN, STAGES>(sched, ws, tickets, err, timeout, 0, 0);
 }
 
@@ -1291,8 +1402,7 @@ static const TileKernel& tile_kernel(int tile) {
 // Grouped launches come in eleven kernel families: the eight 1-CTA tiles, then the
 // cta_group::2 forms of the pair tiles (256x128, 256x256, 256x192).
 constexpr int kGroupFamilies = RG_NUM_TILES + RG_NUM_PAIR_TILES;
-using GroupedFn = void (*)(const GroupHeader*, const GroupItem*, const CUtensorMap, float*, int32_t*, int32_t*,
-                           long long);
+using GroupedFn = void (*)(const GroupHeader*, const CUtensorMap, float*, int32_t*, int32_t*, long long);
 static const void* grouped_kernel(int family) {
   static const GroupedFn table[kGroupFamilies] = {
       gemm_bf16_grouped_kernel<128, 64, 8>,  gemm_bf16_grouped_kernel<128, 128, 6>,
@@ -2131,7 +2241,7 @@ struct rg_group {
 
 namespace rg {
 static_assert(sizeof(GroupHeader) == 128 && sizeof(GroupItem) == 512, "work-list record sizes");
-static size_t group_bytes(int n) { return sizeof(GroupHeader) + static_cast<size_t>(n) * sizeof(GroupItem); }
+static size_t group_bytes(int n) { return group_items_offset(n) + static_cast<size_t>(n) * sizeof(GroupItem); }
 
 static void group_free(rg_group* g) {
   if (!g) return;
@@ -2158,13 +2268,12 @@ static int group_build_graph(rg_group* g, int family, rg_group::Slot& sl) {
                                cudaMemcpyHostToDevice);
   if (e == cudaSuccess) {
     const GroupHeader* hdr = reinterpret_cast<const GroupHeader*>(sl.dev);
-    const GroupItem* items = reinterpret_cast<const GroupItem*>(sl.dev + sizeof(GroupHeader));
     CUtensorMap tmW = g->fam[family].tmW;
     float* ws = g->ws;
     int32_t* tickets = g->tickets;
     int32_t* err = g->ctx->err;
     long long timeout = g->ctx->timeout;
-    void* params[7] = {&hdr, &items, &tmW, &ws, &tickets, &err, &timeout};
+    void* params[6] = {&hdr, &tmW, &ws, &tickets, &err, &timeout};
     const bool two = family >= RG_NUM_TILES;
     cudaKernelNodeParams kp = {};
     kp.func = const_cast<void*>(grouped_kernel(family));
@@ -2221,8 +2330,10 @@ static int group_flush(rg_group* g, int family, const std::vector<GroupItem>& it
   auto* hdr = reinterpret_cast<GroupHeader*>(sl.host);
   hdr->n_items = static_cast<int32_t>(items.size());
   hdr->total_units = static_cast<int32_t>(units);
-  std::memcpy(sl.host + sizeof(GroupHeader), items.data(), items.size() * sizeof(GroupItem));
   const int n = static_cast<int>(items.size());
+  auto* starts = reinterpret_cast<int32_t*>(sl.host + sizeof(GroupHeader));
+  for (int i = 0; i < n; ++i) starts[i] = items[static_cast<size_t>(i)].unit_start;
+  std::memcpy(sl.host + group_items_offset(n), items.data(), items.size() * sizeof(GroupItem));
   e = cudaGraphExecMemcpyNodeSetParams1D(sl.exec, sl.copy_node, sl.dev, sl.host, group_bytes(n),
                                          cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaGraphLaunch(sl.exec, st);
@@ -2312,9 +2423,15 @@ extern "C" int rg_gemm_grouped(rg_group* g, const rg_group_problem* probs, int32
     if (q.L.zero_only) return rg::fail(RG_ERR_INVALID, "rg_gemm_grouped: K == 0 problems are not grouped");
     prep.push_back(q);
   }
+  // Longest units first: the units are dealt to the CTAs round robin, so each wave then holds
+  // units of about the same length and the last ones are the shortest.
+  std::vector<int32_t> order(prep.size());
+  for (size_t i = 0; i < order.size(); ++i) order[i] = static_cast<int32_t>(i);
+  auto unit_blocks = [&](int32_t i) { return prep[i].L.args.kblocks / prep[i].L.args.splits; };
+  std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return unit_blocks(a) > unit_blocks(b); });
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   std::vector<rg::GroupItem> items;
-  items.reserve(static_cast<size_t>(g->max_items));
+  items.reserve(prep.size());
   for (int f = 0; f < rg::kGroupFamilies; ++f) {
     bool any = false;
     for (const auto& q : prep) any = any || q.family == f;
@@ -2324,15 +2441,27 @@ extern "C" int rg_gemm_grouped(rg_group* g, const rg_group_problem* probs, int32
     const bool two = f >= RG_NUM_TILES;
     const int bm = two ? 128 : rg::tile_kernel(f).bm;
     const int64_t ws_rows = g->ws_bytes / (4 * rg::family_bn(f));
+    // the family's K blocks of its tiles (pair tiles), and the CTAs (clusters) that share them
+    const bool serial_ok = rg::serial_tile(rg::family_bn(f) * (bm / 128));
+    const int64_t clusters = two ? g->ctx->sm_count / 2 : g->ctx->sm_count;
+    int64_t blocks = 0;
+    for (const auto& q : prep)
+      if (q.family == f)
+        blocks += static_cast<int64_t>(q.L.args.tiles_m) * q.L.args.tiles_n / (two ? 2 : 1) * q.L.args.kblocks;
     items.clear();
     int64_t units = 0, rows = 0, tks = 0;
-    for (const auto& q : prep) {
+    for (const int32_t qi : order) {
+      const Prepared& q = prep[static_cast<size_t>(qi)];
       if (q.family != f) continue;
       const rg::GemmArgs& a = q.L.args;
       const int64_t ntiles = static_cast<int64_t>(a.tiles_m) * a.tiles_n;
-      const int64_t my_units = (two ? ntiles / 2 : ntiles) * a.splits;
-      const int64_t my_rows = a.splits > 1 ? a.splits * ntiles * bm : 0;
-      const int64_t my_tks = a.splits > 1 ? 4 * ntiles : 0;
+      // The K splits of a tile as one unit, where that is no longer than a CTA's (cluster's) share of
+      // the family's K blocks: splitting then only adds the partials' traffic, not parallelism.
+      const bool serial = a.splits > 1 && serial_ok && a.kblocks * clusters <= blocks;
+      const int32_t splits = serial ? 1 : a.splits;
+      const int64_t my_units = (two ? ntiles / 2 : ntiles) * splits;
+      const int64_t my_rows = splits > 1 ? splits * ntiles * bm : 0;
+      const int64_t my_tks = splits > 1 ? 4 * ntiles : 0;
       if (my_rows > ws_rows || my_tks > rg::kMaxTickets)
         return rg::fail(RG_ERR_SHAPE, "rg_gemm_grouped: a problem's split-K partials exceed the group's workspace");
       if (static_cast<int>(items.size()) == g->max_items || rows + my_rows > ws_rows || tks + my_tks > rg::kMaxTickets ||
@@ -2353,7 +2482,8 @@ extern "C" int rg_gemm_grouped(rg_group* g, const rg_group_problem* probs, int32
       it.tiles_n = a.tiles_n;
       it.kblocks = a.kblocks;
       it.unit_start = static_cast<int32_t>(units);
-      it.splits = a.splits;
+      it.splits = splits;
+      it.segs = serial ? a.splits : 1;
       it.ws_row0 = static_cast<int32_t>(rows);
       it.tk0 = static_cast<int32_t>(tks);
       items.push_back(it);
