@@ -318,21 +318,24 @@ int rg_surface_stats(const rg_grid* grid, const int64_t* t_ns, double* tflops_ou
  * The problems are sorted into eleven kernel families (the eight 1-CTA tiles, the
  * three cta_group::2 tiles); each family present becomes one persistent launch
  * over all SMs whose work units are the concatenation of its problems'
- * (tile, K split) units.  Each problem has its own sizes, operands, leading
- * dimensions, beta and padded launch extents (pm, pn, pk as in rg_gemm;
- * 0 = no padding).  The split-K partials and tickets live in a workspace the
- * group owns (workspace_bytes, at least 1 MiB); when a family's problems need
- * more than it holds at once, the family runs as several launches in turn.
- * The launches of one call run one after another on `stream`; problems of one
- * call must not write overlapping parts of C (they may run concurrently).
+ * (tile, K split) units, longest first.  Where a family's tiles fill the chip, its
+ * split problems run all K splits of a tile in turn on one CTA (pair) instead (the
+ * 128x64, 128x128, 256x64 tiles and the 256x128 pairs).  Each problem has its own
+ * sizes, operands, leading dimensions, beta and padded launch extents (pm, pn, pk
+ * as in rg_gemm; 0 = no padding).  The split-K partials and tickets live in a
+ * workspace the group owns (workspace_bytes, at least 1 MiB); when the problems
+ * need more than it holds at once, or a family has more than max_items, they run as
+ * several sets of launches in turn.  The launches of one set may run side by side;
+ * problems of one call must not write overlapping parts of C.
  * A result is bitwise that of rg_gemm with the same variant (same split
  * boundaries and summation order), whatever else the call contains.
- * rg_group_create allocates the workspace and tickets and, for each family,
- * kGroupSlots = 4 slots of work lists (pinned host + device, for max_items
- * problems each), instantiating one CUDA graph per slot: [copy the host list
- * to the device list, grouped kernel].  rg_gemm_grouped allocates nothing: it
- * fills the next slot of each family it uses (waiting first until that slot's
- * replay from 4 launches ago has finished), then replays its graph on `stream`;
+ * rg_group_create allocates the workspace and tickets and kGroupSlots = 4 slots of
+ * work lists (pinned host + device, for max_items problems of each family),
+ * instantiating each slot's CUDA graphs: [copy the host list to the device list,
+ * then grouped kernels], one per family and one with all of them.  rg_gemm_grouped
+ * allocates nothing: it fills the next slot (waiting first until that slot's replay
+ * from 4 launches ago has finished) and replays the graph of the one family present,
+ * or that of all with the families present enabled, on `stream`;
  * the call returns without waiting for the GEMMs.  Operand conventions and
  * alignment are those of rg_gemm; every problem is checked before anything is
  * enqueued (RG_ERR_SHAPE for one whose partials alone exceed the workspace);

@@ -511,9 +511,10 @@ struct TwoSmSched {
 // its split-K partials and tickets in the launch's workspace.  TWO_SM: units are
 // (256-row pair tile, split) and every 2-CTA cluster runs one at a time as a
 // tcgen05 cta_group::2 unit (tiles_m counts 128-row tiles).
-// Work-list records keep CUtensorMap's 128-byte alignment: a 128-byte header, the
-// items' first units (4 bytes each, padded to 128 bytes), then 512-byte items (three
-// maps and the sizes).  Finding a unit's item reads the 4-byte array only, 32 entries
+// A work list serves every kernel family of a launch: a 128-byte directory, then a
+// section per family present.  Its records keep CUtensorMap's 128-byte alignment: a
+// 128-byte header, the items' first units (4 bytes each, padded to 128 bytes), then
+// 512-byte items (three maps and the sizes).  Finding a unit's item reads the 4-byte array only, 32 entries
 // to a warp load, from the last unit's item on: a CTA's units ascend.
 struct alignas(128) GroupItem {
   CUtensorMap a, b, c;
@@ -528,6 +529,12 @@ struct alignas(128) GroupHeader {
   int32_t total_units;
   int32_t reserved[30];
 };
+struct alignas(128) GroupDirectory {
+  int64_t bytes;                                      // of the whole list
+  int32_t section[RG_NUM_TILES + RG_NUM_PAIR_TILES];  // of each family, as its offset / 128 (its kernel runs only if present)
+  int32_t reserved[19];
+};
+static_assert(sizeof(GroupDirectory) == 128, "work-list directory");
 __host__ __device__ constexpr size_t group_items_offset(int n) {
   return sizeof(GroupHeader) + (static_cast<size_t>(n) * 4 + 127) / 128 * 128;
 }
@@ -1324,10 +1331,36 @@ __global__ void __launch_bounds__(kThreads, 1)
   gemm_body<128, BN, STAGES>(sched, args.ws, args.tickets, args.err, args.timeout, args.stall, args.early, args.trace);
 }
 
+__device__ __forceinline__ const GroupHeader* group_section(const unsigned char* list, int family) {
+  const int32_t at = reinterpret_cast<const GroupDirectory*>(list)->section[family];
+  return reinterpret_cast<const GroupHeader*>(list + static_cast<size_t>(at) * 128);
+}
+
+// Copies a work list from pinned host memory, where its directory gives its bytes; the first pass over
+// the grid does not wait for them (it stays inside the list's buffers, `capacity` bytes, a multiple of 16).
+// A copy by the SMs rather than by a copy engine: no hand-over between engines, nothing in the graph to
+// update for each call, and the grouped kernels start while it runs (a programmatic edge).  One problem of
+// 128^3 alone: 13.4 us with a copy node, 11.3 so; 24 problems in five families 80.4 and 76.7.
+constexpr int kCopyCtas = 8, kCopyThreads = 512;
+__global__ void __launch_bounds__(kCopyThreads) group_copy_kernel(const uint4* __restrict__ host, uint4* __restrict__ dev,
+                                                                  int64_t capacity) {
+  const int64_t step = static_cast<int64_t>(kCopyCtas) * kCopyThreads;
+  int64_t i = static_cast<int64_t>(blockIdx.x) * kCopyThreads + threadIdx.x;
+  grid_launch_dependents();
+  const int64_t bytes = *reinterpret_cast<const volatile int64_t*>(host);
+  if (i < capacity / 16) dev[i] = host[i];
+  const int64_t n = (bytes + 15) / 16;
+  for (i += step; i < n; i += step) dev[i] = host[i];
+}
+
 template <int BM, int BN, int STAGES>
 __global__ void __launch_bounds__(kThreads, 1)
-    gemm_bf16_grouped_kernel(const GroupHeader* __restrict__ hdr, const __grid_constant__ CUtensorMap tmW, float* ws,
-                             int32_t* tickets, int32_t* err, long long timeout) {
+    gemm_bf16_grouped_kernel(const unsigned char* __restrict__ list, int family,
+                             const __grid_constant__ CUtensorMap tmW, float* ws, int32_t* tickets, int32_t* err,
+                             long long timeout) {
+  grid_dependency_wait();  // the list has been copied
+  const GroupHeader* hdr = group_section(list, family);
+  if (static_cast<int>(blockIdx.x) >= hdr->total_units) return;  // no unit for this CTA: the SM is another family's
   GroupSched<false> sched{hdr, &tmW};
   gemm_body<BM, BN, STAGES>(sched, ws, tickets, err, timeout, 0, 0);
 }
@@ -1336,8 +1369,12 @@ __global__ void __launch_bounds__(kThreads, 1)
 // two CTAs, so a graph kernel node launches it as pairs without a launch attribute.
 template <int BN, int STAGES>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-    gemm_bf16_grouped_2sm_kernel(const GroupHeader* __restrict__ hdr, const __grid_constant__ CUtensorMap tmW,
-                                 float* ws, int32_t* tickets, int32_t* err, long long timeout) {
+    gemm_bf16_grouped_2sm_kernel(const unsigned char* __restrict__ list, int family,
+                                 const __grid_constant__ CUtensorMap tmW, float* ws, int32_t* tickets, int32_t* err,
+                                 long long timeout) {
+  grid_dependency_wait();  // the list has been copied
+  const GroupHeader* hdr = group_section(list, family);
+  if (static_cast<int>(blockIdx.x) / 2 >= hdr->total_units) return;  // both CTAs of the cluster
   GroupSched<true> sched{hdr, &tmW};
   gemm_body<128, BN, STAGES>(sched, ws, tickets, err, timeout, 0, 0);
 }
@@ -1402,7 +1439,7 @@ static const TileKernel& tile_kernel(int tile) {
 // Grouped launches come in eleven kernel families: the eight 1-CTA tiles, then the
 // cta_group::2 forms of the pair tiles (256x128, 256x256, 256x192).
 constexpr int kGroupFamilies = RG_NUM_TILES + RG_NUM_PAIR_TILES;
-using GroupedFn = void (*)(const GroupHeader*, const CUtensorMap, float*, int32_t*, int32_t*, long long);
+using GroupedFn = void (*)(const unsigned char*, int, const CUtensorMap, float*, int32_t*, int32_t*, long long);
 static const void* grouped_kernel(int family) {
   static const GroupedFn table[kGroupFamilies] = {
       gemm_bf16_grouped_kernel<128, 64, 8>,  gemm_bf16_grouped_kernel<128, 128, 6>,
@@ -2200,16 +2237,22 @@ extern "C" int rg_gemm_memtwin(rg_ctx* ctx, int64_t M, int64_t N, int64_t K, con
 
 // ------------------------------------------------------------------ grouped GEMM under CUDA graphs
 //
-// A group object owns, per kernel family, kGroupSlots slots (built on the
-// family's first use).  Each slot: a pinned host work list, a device work list
-// (header + items), a CUDA graph [copy host list -> device list, persistent
-// grouped kernel over all SMs] instantiated once, and an event marking the
-// slot's last replay.  A call sorts its problems by family; for each family
-// present it fills work lists -- starting a further list whenever the next item's
-// split-K partials or tickets would not fit the group's workspace, or the list is
-// full -- and replays one graph per list on the caller's stream, so the lists of
-// one call run one after another and each may reuse the whole workspace.  The
-// graph's topology never changes; only the list contents do.
+// A group object owns kGroupSlots slots.  Each slot: a pinned host work list, a device
+// work list, CUDA graphs instantiated once, and an event marking the slot's last replay.
+// A graph is [copy host list -> device list, then grouped kernels, each on the copy alone]:
+// one graph per kernel family, and one with all of them, of which a replay enables those
+// present.  A call sorts its problems into the families' sections of one work list --
+// starting a further list whenever the next item's split-K partials or tickets would not
+// fit the group's workspace next to the list's others, or the list holds max_items of its
+// family -- and replays, on the caller's stream, the graph of the one family present, or
+// the graph of all.  The kernels of a list may run side by side (their problems are
+// independent and their parts of the workspace disjoint): a family's CTAs take the SMs
+// that another's leave, where a graph per family ran them one after another, each with a
+// copy, a start and a tail of its own (48 mixed problems in two families 60.6 -> 52.1 us,
+// 24 of up to 4096 in five 110 -> 79).  A disabled node is not free (about 0.5 us each), so
+// a call of one family, the common one, has its own graph (8 problems: 13.7 -> 10.7 us).
+// The lists of one call run in turn, so each may use the whole workspace.  The graphs'
+// topology never changes; only the list contents and the enabled nodes do.
 namespace rg {
 constexpr int kGroupSlots = 4;
 constexpr int64_t kGroupMinWorkspace = 1 << 20;
@@ -2222,125 +2265,176 @@ struct rg_group {
   float* ws = nullptr;
   int64_t ws_bytes = 0;
   int32_t* tickets = nullptr;
+  int64_t list_bytes = 0;  // capacity of a work list
   struct Slot {
-    unsigned char* host = nullptr;  // pinned: header + items
+    unsigned char* host = nullptr;  // pinned
     unsigned char* dev = nullptr;
+    // [copy, one family's kernel] for each family, and [copy, every family's kernel side by side]
+    cudaGraphExec_t one[rg::kGroupFamilies] = {};
     cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
-    cudaGraphNode_t copy_node = nullptr;
+    cudaGraphExec_t all = nullptr;
+    cudaGraphNode_t kernel[rg::kGroupFamilies] = {};  // of `all`
+    uint32_t enabled = 0;  // families whose kernel nodes of `all` are enabled
     cudaEvent_t done = nullptr;
     bool used = false;
-  };
-  struct Family {
-    Slot slot[rg::kGroupSlots];
-    int next = 0;
-    bool ready = false;
-    CUtensorMap tmW;
-  } fam[rg::kGroupFamilies];
+  } slot[rg::kGroupSlots];
+  int next = 0;
 };
 
 namespace rg {
 static_assert(sizeof(GroupHeader) == 128 && sizeof(GroupItem) == 512, "work-list record sizes");
-static size_t group_bytes(int n) { return group_items_offset(n) + static_cast<size_t>(n) * sizeof(GroupItem); }
+// Bytes of a family's section of n items, and of a list of n items in each family.
+static size_t section_bytes(int n) { return group_items_offset(n) + static_cast<size_t>(n) * sizeof(GroupItem); }
+static size_t group_bytes(int n) { return sizeof(GroupDirectory) + kGroupFamilies * section_bytes(n); }
 
 static void group_free(rg_group* g) {
   if (!g) return;
-  for (auto& f : g->fam)
-    for (auto& sl : f.slot) {
-      if (sl.used) cudaEventSynchronize(sl.done);
-      if (sl.exec) cudaGraphExecDestroy(sl.exec);
-      if (sl.graph) cudaGraphDestroy(sl.graph);
-      if (sl.done) cudaEventDestroy(sl.done);
-      if (sl.host) cudaFreeHost(sl.host);
-      if (sl.dev) cudaFree(sl.dev);
-    }
+  for (auto& sl : g->slot) {
+    if (sl.used) cudaEventSynchronize(sl.done);
+    for (auto exec : sl.one)
+      if (exec) cudaGraphExecDestroy(exec);
+    if (sl.all) cudaGraphExecDestroy(sl.all);
+    if (sl.graph) cudaGraphDestroy(sl.graph);
+    if (sl.done) cudaEventDestroy(sl.done);
+    if (sl.host) cudaFreeHost(sl.host);
+    if (sl.dev) cudaFree(sl.dev);
+  }
   cudaFree(g->ws);
   cudaFree(g->tickets);
   delete g;
 }
 
-static int group_build_graph(rg_group* g, int family, rg_group::Slot& sl) {
-  cudaGraph_t graph = nullptr;
-  cudaError_t e = cudaGraphCreate(&graph, 0);
-  if (e != cudaSuccess) return cuda_fail(e, "rg_group: graph");
-  cudaGraphNode_t copy = nullptr, kern = nullptr;
-  e = cudaGraphAddMemcpyNode1D(&copy, graph, nullptr, 0, sl.dev, sl.host, group_bytes(g->max_items),
-                               cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) {
-    const GroupHeader* hdr = reinterpret_cast<const GroupHeader*>(sl.dev);
-    CUtensorMap tmW = g->fam[family].tmW;
+// Adds a slot's copy and the kernels of `families` (a bit mask), each after the copy, to a graph.
+static int group_add_nodes(rg_group* g, rg_group::Slot& sl, cudaGraph_t graph, uint32_t families,
+                           cudaGraphNode_t* kernels) {
+  const uint4* host = reinterpret_cast<const uint4*>(sl.host);
+  uint4* dev = reinterpret_cast<uint4*>(sl.dev);
+  int64_t capacity = g->list_bytes;
+  void* copy_params[3] = {&host, &dev, &capacity};
+  cudaKernelNodeParams kc = {};
+  kc.func = reinterpret_cast<void*>(group_copy_kernel);
+  kc.gridDim = dim3(kCopyCtas);
+  kc.blockDim = dim3(kCopyThreads);
+  kc.kernelParams = copy_params;
+  cudaGraphNode_t copy = nullptr;
+  cudaError_t e = cudaGraphAddKernelNode(&copy, graph, nullptr, 0, &kc);
+  for (int f = 0; f < kGroupFamilies && e == cudaSuccess; ++f) {
+    if (!(families >> f & 1)) continue;
+    const int bn = family_bn(f);
+    CUtensorMap tmW;
+    const int rc = make_map(&tmW, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, g->ws, static_cast<uint64_t>(bn),
+                            static_cast<uint64_t>(g->ws_bytes / (4 * bn)), static_cast<uint64_t>(bn) * 4, 32, 32);
+    if (rc != RG_OK) return rc;
+    const unsigned char* list = sl.dev;
     float* ws = g->ws;
     int32_t* tickets = g->tickets;
     int32_t* err = g->ctx->err;
     long long timeout = g->ctx->timeout;
-    void* params[6] = {&hdr, &tmW, &ws, &tickets, &err, &timeout};
-    const bool two = family >= RG_NUM_TILES;
+    void* params[7] = {&list, &f, &tmW, &ws, &tickets, &err, &timeout};
+    const bool two = f >= RG_NUM_TILES;
     cudaKernelNodeParams kp = {};
-    kp.func = const_cast<void*>(grouped_kernel(family));
+    kp.func = const_cast<void*>(grouped_kernel(f));
     kp.gridDim = dim3(static_cast<unsigned>(two ? g->ctx->sm_count / 2 * 2 : g->ctx->sm_count));
     kp.blockDim = dim3(kThreads);
-    kp.sharedMemBytes = static_cast<unsigned>(family_smem(family));
+    kp.sharedMemBytes = static_cast<unsigned>(family_smem(f));
     kp.kernelParams = params;
-    e = cudaGraphAddKernelNode(&kern, graph, &copy, 1, &kp);
+    e = cudaGraphAddKernelNode(&kernels[f], graph, nullptr, 0, &kp);
+    if (e == cudaSuccess) {  // started while the copy runs; it waits for the copy's end before reading the list
+      cudaGraphEdgeData edge = {};
+      edge.from_port = cudaGraphKernelNodePortProgrammatic;
+      edge.type = cudaGraphDependencyTypeProgrammatic;
+      e = cudaGraphAddDependencies(graph, &copy, &kernels[f], &edge, 1);
+    }
   }
-  if (e == cudaSuccess) e = cudaGraphInstantiate(&sl.exec, graph, 0);
-  if (e != cudaSuccess) {
-    cudaGraphDestroy(graph);
-    return cuda_fail(e, "rg_group: build graph");
-  }
-  sl.graph = graph;
-  sl.copy_node = copy;
-  return RG_OK;
+  return e == cudaSuccess ? RG_OK : cuda_fail(e, "rg_group: graph nodes");
 }
 
-// Slots, graphs and the workspace tensor map of one family, on its first use.
-static int group_family_ready(rg_group* g, int family) {
-  rg_group::Family& f = g->fam[family];
-  if (f.ready) return RG_OK;
-  const int bn = family_bn(family);
-  int rc = make_map(&f.tmW, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, g->ws, static_cast<uint64_t>(bn),
-                    static_cast<uint64_t>(g->ws_bytes / (4 * bn)), static_cast<uint64_t>(bn) * 4, 32, 32);
-  if (rc != RG_OK) return rc;
-  const size_t bytes = group_bytes(g->max_items);
-  for (auto& sl : f.slot) {
-    cudaError_t e = cudaMallocHost(&sl.host, bytes);
-    if (e == cudaSuccess) e = cudaMalloc(&sl.dev, bytes);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      return fail(RG_ERR_OOM, std::string("rg_gemm_grouped: work lists: ") + cudaGetErrorString(e));
-    }
-    std::memset(sl.host, 0, bytes);
-    rc = group_build_graph(g, family, sl);
+// A slot's work lists and graphs.
+static int group_slot_init(rg_group* g, rg_group::Slot& sl) {
+  const size_t bytes = static_cast<size_t>(g->list_bytes);
+  cudaError_t e = cudaMallocHost(&sl.host, bytes);
+  if (e == cudaSuccess) e = cudaMalloc(&sl.dev, bytes);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return fail(RG_ERR_OOM, std::string("rg_group_create: work lists: ") + cudaGetErrorString(e));
+  }
+  std::memset(sl.host, 0, bytes);
+  for (int f = 0; f < kGroupFamilies; ++f) {
+    cudaGraph_t graph = nullptr;
+    cudaGraphNode_t unused[kGroupFamilies];
+    if ((e = cudaGraphCreate(&graph, 0)) != cudaSuccess) return cuda_fail(e, "rg_group: graph");
+    int rc = group_add_nodes(g, sl, graph, 1u << f, unused);
+    if (rc == RG_OK && (e = cudaGraphInstantiate(&sl.one[f], graph, 0)) != cudaSuccess)
+      rc = cuda_fail(e, "rg_group: build graph");
+    cudaGraphDestroy(graph);
     if (rc != RG_OK) return rc;
   }
-  f.ready = true;
-  return RG_OK;
+  if ((e = cudaGraphCreate(&sl.graph, 0)) != cudaSuccess) return cuda_fail(e, "rg_group: graph");
+  const int rc = group_add_nodes(g, sl, sl.graph, (1u << kGroupFamilies) - 1, sl.kernel);
+  if (rc != RG_OK) return rc;
+  e = cudaGraphInstantiate(&sl.all, sl.graph, 0);
+  for (int f = 0; f < kGroupFamilies && e == cudaSuccess; ++f) e = cudaGraphNodeSetEnabled(sl.all, sl.kernel[f], 0);
+  return e == cudaSuccess ? RG_OK : cuda_fail(e, "rg_group: build graph");
 }
 
-// Replays the next slot of `family` with the list in `items` (count items, units units).
-static int group_flush(rg_group* g, int family, const std::vector<GroupItem>& items, int64_t units,
-                       cudaStream_t st) {
-  if (items.empty()) return RG_OK;
-  rg_group::Family& f = g->fam[family];
-  rg_group::Slot& sl = f.slot[f.next];
-  f.next = (f.next + 1) % kGroupSlots;
+// The items of one work list, by family.
+struct GroupList {
+  std::vector<GroupItem> items[kGroupFamilies];
+  int64_t units[kGroupFamilies] = {};
+  int64_t ws_bytes = 0, tickets = 0;  // of the workspace and tickets its items use
+  int count = 0;
+  void clear() {
+    for (int f = 0; f < kGroupFamilies; ++f) {
+      items[f].clear();
+      units[f] = 0;
+    }
+    ws_bytes = tickets = 0;
+    count = 0;
+  }
+};
+
+// Replays the next slot with the list.
+static int group_flush(rg_group* g, const GroupList& list, cudaStream_t st) {
+  if (list.count == 0) return RG_OK;
+  rg_group::Slot& sl = g->slot[g->next];
+  g->next = (g->next + 1) % kGroupSlots;
   cudaError_t e;
   if (sl.used && (e = cudaEventSynchronize(sl.done)) != cudaSuccess) return cuda_fail(e, "rg_gemm_grouped: slot");
-  auto* hdr = reinterpret_cast<GroupHeader*>(sl.host);
-  hdr->n_items = static_cast<int32_t>(items.size());
-  hdr->total_units = static_cast<int32_t>(units);
-  const int n = static_cast<int>(items.size());
-  auto* starts = reinterpret_cast<int32_t*>(sl.host + sizeof(GroupHeader));
-  for (int i = 0; i < n; ++i) starts[i] = items[static_cast<size_t>(i)].unit_start;
-  std::memcpy(sl.host + group_items_offset(n), items.data(), items.size() * sizeof(GroupItem));
-  e = cudaGraphExecMemcpyNodeSetParams1D(sl.exec, sl.copy_node, sl.dev, sl.host, group_bytes(n),
-                                         cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaGraphLaunch(sl.exec, st);
+  auto* dir = reinterpret_cast<GroupDirectory*>(sl.host);
+  size_t at = sizeof(GroupDirectory);
+  uint32_t present = 0;
+  int kernels = 0;
+  for (int f = 0; f < kGroupFamilies; ++f) {
+    const std::vector<GroupItem>& items = list.items[f];
+    if (items.empty()) continue;
+    present |= 1u << f;
+    ++kernels;
+    const int n = static_cast<int>(items.size());
+    dir->section[f] = static_cast<int32_t>(at / 128);
+    auto* hdr = reinterpret_cast<GroupHeader*>(sl.host + at);
+    hdr->n_items = n;
+    hdr->total_units = static_cast<int32_t>(list.units[f]);
+    auto* starts = reinterpret_cast<int32_t*>(hdr + 1);
+    for (int i = 0; i < n; ++i) starts[i] = items[static_cast<size_t>(i)].unit_start;
+    std::memcpy(sl.host + at + group_items_offset(n), items.data(), items.size() * sizeof(GroupItem));
+    at += section_bytes(n);
+  }
+  dir->bytes = static_cast<int64_t>(at);
+  cudaGraphExec_t exec = sl.all;
+  for (int f = 0; f < kGroupFamilies; ++f) {
+    if (present == 1u << f) exec = sl.one[f];
+    if (kernels > 1 && ((present ^ sl.enabled) >> f & 1)) {
+      if ((e = cudaGraphNodeSetEnabled(sl.all, sl.kernel[f], present >> f & 1)) != cudaSuccess)
+        return cuda_fail(e, "rg_gemm_grouped: graph node");
+      sl.enabled ^= 1u << f;
+    }
+  }
+  e = cudaGraphLaunch(exec, st);
   if (e == cudaSuccess) e = cudaEventRecord(sl.done, st);
   if (e != cudaSuccess) return cuda_fail(e, "rg_gemm_grouped: replay");
   sl.used = true;
-  g->ctx->launches += 1;
+  g->ctx->launches += kernels;
   return RG_OK;
 }
 }  // namespace rg
@@ -2367,10 +2461,11 @@ extern "C" int rg_group_create(rg_ctx* ctx, int32_t tile, int32_t max_items, int
     rg::group_free(g);
     return rg::fail(RG_ERR_OOM, std::string("rg_group_create: ") + cudaGetErrorString(e));
   }
-  // every family's work lists and graphs now, so that no call allocates or
-  // instantiates on the serving path
-  for (int f = 0; f < rg::kGroupFamilies; ++f) {
-    const int rc = rg::group_family_ready(g, f);
+  // every slot's lists and graph now, so that no call allocates or instantiates on the
+  // serving path
+  g->list_bytes = static_cast<int64_t>(rg::group_bytes(max_items));
+  for (auto& sl : g->slot) {
+    const int rc = rg::group_slot_init(g, sl);
     if (rc != RG_OK) {
       rg::group_free(g);
       return rc;
@@ -2429,71 +2524,70 @@ extern "C" int rg_gemm_grouped(rg_group* g, const rg_group_problem* probs, int32
   for (size_t i = 0; i < order.size(); ++i) order[i] = static_cast<int32_t>(i);
   auto unit_blocks = [&](int32_t i) { return prep[i].L.args.kblocks / prep[i].L.args.splits; };
   std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return unit_blocks(a) > unit_blocks(b); });
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  std::vector<rg::GroupItem> items;
-  items.reserve(prep.size());
-  for (int f = 0; f < rg::kGroupFamilies; ++f) {
-    bool any = false;
-    for (const auto& q : prep) any = any || q.family == f;
-    if (!any) continue;
-    int rc = rg::group_family_ready(g, f);
-    if (rc != RG_OK) return rc;
-    const bool two = f >= RG_NUM_TILES;
-    const int bm = two ? 128 : rg::tile_kernel(f).bm;
-    const int64_t ws_rows = g->ws_bytes / (4 * rg::family_bn(f));
-    // the family's K blocks of its tiles (pair tiles), and the CTAs (clusters) that share them
-    const bool serial_ok = rg::serial_tile(rg::family_bn(f) * (bm / 128));
-    const int64_t clusters = two ? g->ctx->sm_count / 2 : g->ctx->sm_count;
-    int64_t blocks = 0;
-    for (const auto& q : prep)
-      if (q.family == f)
-        blocks += static_cast<int64_t>(q.L.args.tiles_m) * q.L.args.tiles_n / (two ? 2 : 1) * q.L.args.kblocks;
-    items.clear();
-    int64_t units = 0, rows = 0, tks = 0;
-    for (const int32_t qi : order) {
-      const Prepared& q = prep[static_cast<size_t>(qi)];
-      if (q.family != f) continue;
-      const rg::GemmArgs& a = q.L.args;
-      const int64_t ntiles = static_cast<int64_t>(a.tiles_m) * a.tiles_n;
-      // The K splits of a tile as one unit, where that is no longer than a CTA's (cluster's) share of
-      // the family's K blocks: splitting then only adds the partials' traffic, not parallelism.
-      const bool serial = a.splits > 1 && serial_ok && a.kblocks * clusters <= blocks;
-      const int32_t splits = serial ? 1 : a.splits;
-      const int64_t my_units = (two ? ntiles / 2 : ntiles) * splits;
-      const int64_t my_rows = splits > 1 ? splits * ntiles * bm : 0;
-      const int64_t my_tks = splits > 1 ? 4 * ntiles : 0;
-      if (my_rows > ws_rows || my_tks > rg::kMaxTickets)
-        return rg::fail(RG_ERR_SHAPE, "rg_gemm_grouped: a problem's split-K partials exceed the group's workspace");
-      if (static_cast<int>(items.size()) == g->max_items || rows + my_rows > ws_rows || tks + my_tks > rg::kMaxTickets ||
-          units + my_units > (1LL << 30)) {
-        if ((rc = rg::group_flush(g, f, items, units, st)) != RG_OK) return rc;
-        items.clear();
-        units = rows = tks = 0;
-      }
-      rg::GroupItem it;
-      std::memset(&it, 0, sizeof(it));
-      it.a = q.L.a;
-      it.b = q.L.b;
-      it.c = q.L.c;
-      it.M = a.M;
-      it.N = a.N;
-      it.beta = a.beta;
-      it.tiles_m = a.tiles_m;
-      it.tiles_n = a.tiles_n;
-      it.kblocks = a.kblocks;
-      it.unit_start = static_cast<int32_t>(units);
-      it.splits = splits;
-      it.segs = serial ? a.splits : 1;
-      it.ws_row0 = static_cast<int32_t>(rows);
-      it.tk0 = static_cast<int32_t>(tks);
-      items.push_back(it);
-      units += my_units;
-      rows += my_rows;
-      tks += my_tks;
-    }
-    if ((rc = rg::group_flush(g, f, items, units, st)) != RG_OK) return rc;
+  // Each family's K blocks over its tiles (pair tiles), and the CTAs (clusters) that share them.
+  int64_t blocks[rg::kGroupFamilies] = {};
+  auto sharers = [&](int f) -> int64_t { return f >= RG_NUM_TILES ? g->ctx->sm_count / 2 : g->ctx->sm_count; };
+  for (const auto& q : prep)
+    blocks[q.family] += static_cast<int64_t>(q.L.args.tiles_m) * q.L.args.tiles_n / (q.family >= RG_NUM_TILES ? 2 : 1) *
+                        q.L.args.kblocks;
+  auto cta_rows = [](int f) { return f >= RG_NUM_TILES ? 128 : rg::tile_kernel(f).bm; };
+  // The K splits of a tile as one unit, where that is no longer than a CTA's (cluster's) share of
+  // the family's K blocks: splitting then only adds the partials' traffic, not parallelism.
+  auto serial_splits = [&](const Prepared& q) {
+    return q.L.args.splits > 1 && rg::serial_tile(rg::family_bn(q.family) * (cta_rows(q.family) / 128)) &&
+           q.L.args.kblocks * sharers(q.family) <= blocks[q.family];
+  };
+  for (const auto& q : prep) {  // partials and tickets of the other splits
+    const int64_t ntiles = static_cast<int64_t>(q.L.args.tiles_m) * q.L.args.tiles_n;
+    if (q.L.args.splits > 1 && !serial_splits(q) &&
+        (q.L.args.splits * ntiles * cta_rows(q.family) > g->ws_bytes / (4LL * rg::family_bn(q.family)) ||
+         4 * ntiles > rg::kMaxTickets))
+      return rg::fail(RG_ERR_SHAPE, "rg_gemm_grouped: a problem's split-K partials exceed the group's workspace");
   }
-  return RG_OK;
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  rg::GroupList list;
+  for (const int32_t qi : order) {
+    const Prepared& q = prep[static_cast<size_t>(qi)];
+    const int f = q.family;
+    const rg::GemmArgs& a = q.L.args;
+    const int bn = rg::family_bn(f), bm = cta_rows(f);
+    const int64_t ntiles = static_cast<int64_t>(a.tiles_m) * a.tiles_n;
+    const bool serial = serial_splits(q);
+    const int32_t splits = serial ? 1 : a.splits;
+    const int64_t my_units = (f >= RG_NUM_TILES ? ntiles / 2 : ntiles) * splits;
+    const int64_t row_bytes = 4LL * bn, my_rows = splits > 1 ? splits * ntiles * bm : 0;
+    const int64_t my_tks = splits > 1 ? 4 * ntiles : 0;
+    int64_t row0 = (list.ws_bytes + row_bytes - 1) / row_bytes;  // the family's workspace rows are row_bytes long
+    if (static_cast<int>(list.items[f].size()) == g->max_items || (my_rows > 0 && (row0 + my_rows) * row_bytes > g->ws_bytes) ||
+        list.tickets + my_tks > rg::kMaxTickets || list.units[f] + my_units > (1LL << 30)) {
+      const int rc = rg::group_flush(g, list, st);
+      if (rc != RG_OK) return rc;
+      list.clear();
+      row0 = 0;
+    }
+    rg::GroupItem it;
+    std::memset(&it, 0, sizeof(it));
+    it.a = q.L.a;
+    it.b = q.L.b;
+    it.c = q.L.c;
+    it.M = a.M;
+    it.N = a.N;
+    it.beta = a.beta;
+    it.tiles_m = a.tiles_m;
+    it.tiles_n = a.tiles_n;
+    it.kblocks = a.kblocks;
+    it.unit_start = static_cast<int32_t>(list.units[f]);
+    it.splits = splits;
+    it.segs = serial ? a.splits : 1;
+    it.ws_row0 = static_cast<int32_t>(my_rows > 0 ? row0 : 0);
+    it.tk0 = static_cast<int32_t>(list.tickets);
+    list.items[f].push_back(it);
+    list.units[f] += my_units;
+    if (my_rows > 0) list.ws_bytes = (row0 + my_rows) * row_bytes;
+    list.tickets += my_tks;
+    ++list.count;
+  }
+  return rg::group_flush(g, list, st);
 }
 
 // ------------------------------------------------------------------ entry point without allocation
