@@ -105,7 +105,7 @@ struct GemmArgs {
   int32_t dp_tiles;         // stream-K: tiles run whole before the shared tail
   int32_t panel;            // tile order: column panels of this many tiles (pairs: tile columns)
   int32_t early;            // 1: A and B are static, so loads may start before the preceding grid completes
-  int32_t reserved_;
+  int32_t whole;            // (pair) tiles run whole, the rest as two half-width units each (see tail_tiles)
   float* ws;                // split-K partials [split][tile][BM][BN]
   int32_t* tickets;         // [tile][4], zero between launches
   int32_t* err;
@@ -134,6 +134,9 @@ struct KCfg {
   static constexpr int SMEM_BYTES = 1024 + BAR_OFF + 256;
   static_assert((2 * STAGES + 9) * 8 <= 256, "barrier block");
   static constexpr uint32_t IDESC = instr_desc(1, 1, 0, 1, 128 * CTAS, BN);
+  // Tiles whose columns can be halved in whole 64-column boxes per CTA (tail tiles).
+  static constexpr bool HALVABLE = BN % (128 * CTAS) == 0;
+  static constexpr uint32_t IDESC_HALF = instr_desc(1, 1, 0, 1, 128 * CTAS, HALVABLE ? BN / 2 : BN);
   static_assert(A_BYTES % 1024 == 0 && B_BYTES % 1024 == 0, "stages must keep 1024-byte alignment");
   static_assert(SMEM_BYTES <= 232448, "shared memory budget");
   static_assert(BN % 64 == 0 && BN <= 256 && (BM == 128 || BM == 256), "tile shape");
@@ -230,6 +233,8 @@ struct Unit {
   int tile, ntiles;  // tile id / tile count of the problem (split-K workspace and tickets)
   int ws_row0 = 0;   // first workspace row of the problem's partials (grouped launches)
   int tk0 = 0;       // first ticket of the problem (grouped launches)
+  bool half = false; // the unit is half of its tile's columns (tail tiles),
+  int noff = 0;      // the left (0) or the right (1) one
   int segs = 1;      // > 1: this unit runs all K splits of its tile, one accumulator after another (grouped launches)
 };
 
@@ -276,18 +281,21 @@ __device__ __forceinline__ Unit split_unit(const CUtensorMap* a, const CUtensorM
 // One problem whose tensor maps are kernel parameters (rg_gemm).  SPLIT: the
 // instance for split-K launches (S > 1); without it the kernel carries no
 // reduction path (and none of its register pressure).
-template <bool SPLIT>
+// TAIL: tiles from `whole` on run as two half-width units each (see tail_tiles).
+template <bool SPLIT, bool TAIL = false>
 struct SingleSched {
   static constexpr bool kMapsInGlobal = false;
   static constexpr bool kMemOnly = false;
   static constexpr bool k2Sm = false;
   static constexpr bool kSplit = SPLIT;
+  static constexpr bool kTail = TAIL;
   static constexpr int rank = 0;
   const CUtensorMap* a;
   const CUtensorMap* b;
   const CUtensorMap* c;
   const CUtensorMap* w;
   int tiles_m, tiles_n, splits, kblocks, M, N, beta;
+  int whole = 0;
   int panel = 1 << 30;
   __device__ __forceinline__ void prefetch() const {
     prefetch_tmap(a);
@@ -295,22 +303,30 @@ struct SingleSched {
     prefetch_tmap(c);
   }
   __device__ __forceinline__ void init() {}
-  // units u = blockIdx.x + i * gridDim.x of the (tile, split) space
+  // units u = blockIdx.x + i * gridDim.x of the (tile, split) space; whole tiles, then halves
   __device__ __forceinline__ int count() const {
-    const int t = tiles_m * tiles_n * splits;
+    int t = tiles_m * tiles_n * splits;
+    if constexpr (TAIL) t += t - whole;
     return static_cast<int>(blockIdx.x) < t ? (t - 1 - static_cast<int>(blockIdx.x)) / static_cast<int>(gridDim.x) + 1
                                             : 0;
   }
   __device__ __forceinline__ Unit unit(int i) const {
-    return split_unit(a, b, c, w, static_cast<int>(blockIdx.x) + i * static_cast<int>(gridDim.x), tiles_m, tiles_n,
-                      splits, kblocks, M, N, beta, panel);
+    const int u = static_cast<int>(blockIdx.x) + i * static_cast<int>(gridDim.x);
+    const int h = TAIL ? max(u - whole, 0) : 0;  // 2 x the tile's place in the tail + the half
+    Unit x = split_unit(a, b, c, w, u - (h + 1) / 2, tiles_m, tiles_n, splits, kblocks, M, N, beta, panel);
+    if constexpr (TAIL) {
+      x.half = u >= whole;
+      x.noff = h & 1;
+    }
+    return x;
   }
 };
 
 // The memory twin of SingleSched: the same units, loads and stores, with the
 // MMAs replaced by no-ops (the memory surface of the four-surface decomposition,
 // Sec. 4).  Its output is whatever the accumulators held: timing only.
-struct MemTwinSched : SingleSched<false> {
+template <bool TAIL>
+struct MemTwinSched : SingleSched<false, TAIL> {
   static constexpr bool kMemOnly = true;
 };
 
@@ -332,6 +348,11 @@ template <class S, class = void>
 struct IsClusterSplit : std::false_type {};
 template <class S>
 struct IsClusterSplit<S, std::void_t<decltype(S::kClusterSplit)>> : std::bool_constant<S::kClusterSplit> {};
+
+template <class S, class = void>
+struct HasTail : std::false_type {};
+template <class S>
+struct HasTail<S, std::void_t<decltype(S::kTail)>> : std::bool_constant<S::kTail> {};
 
 // Stream-K (hybrid): whole waves of tiles run data-parallel, one tile per CTA
 // per wave (tile g + i * G on CTA g, for tiles below dp_tiles: all whole waves,
@@ -449,12 +470,14 @@ struct StreamKSched {
 // memory, and the even CTA issues the MMAs for both.  A CTA whose rows fall
 // outside the problem still loads (zero-filled reads) so that the pair's MMAs
 // are fed; its stores are dropped.  Units are (pair tile, K split).
-template <bool SPLIT>
+// TAIL as for SingleSched, over pair tiles.
+template <bool SPLIT, bool TAIL = false>
 struct TwoSmSched {
   static constexpr bool kMapsInGlobal = false;
   static constexpr bool kMemOnly = false;
   static constexpr bool k2Sm = true;
   static constexpr bool kSplit = SPLIT;
+  static constexpr bool kTail = TAIL;
   const CUtensorMap* a;
   const CUtensorMap* b;
   const CUtensorMap* c;
@@ -462,6 +485,7 @@ struct TwoSmSched {
   int tiles_m, tiles_n, kblocks, M, N, beta;  // tiles_m counts 128-row tiles
   int rank = 0, cid = 0, ncl = 1, pairs = 0;
   int splits = 1;
+  int whole = 0;
   int panel = 1 << 30;
   __device__ __forceinline__ void prefetch() const {
     prefetch_tmap(a);
@@ -475,11 +499,14 @@ struct TwoSmSched {
     pairs = ((tiles_m + 1) / 2) * tiles_n;
   }
   __device__ __forceinline__ int count() const {
-    const int units = pairs * splits;
+    int units = pairs * splits;
+    if constexpr (TAIL) units += units - whole;
     return cid < units ? (units - 1 - cid) / ncl + 1 : 0;
   }
   __device__ __forceinline__ Unit unit(int i) const {
-    const int u = cid + i * ncl;
+    const int i0 = cid + i * ncl;
+    const int h = TAIL ? max(i0 - whole, 0) : 0;  // 2 x the tile's place in the tail + the half
+    const int u = i0 - (h + 1) / 2;
     const int p = u / splits;
     Unit x;
     x.a = a;
@@ -499,6 +526,10 @@ struct TwoSmSched {
     x.beta = beta;
     x.ntiles = tiles_m * tiles_n;
     x.tile = x.tm * tiles_n + x.tn;
+    if constexpr (TAIL) {
+      x.half = i0 >= whole;
+      x.noff = h & 1;
+    }
     return x;
   }
 };
@@ -657,6 +688,8 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
   using C = KCfg<BM, BN, STAGES, P2 ? 2 : 1>;
   // units may run all K splits of their tile (a thread then holds its sums of the whole tile in registers)
   constexpr bool SERIAL = Sched::kMapsInGlobal && serial_tile(C::ACC_COLS);
+  constexpr bool TAIL = HasTail<Sched>::value;  // units may be halves of their tile's columns
+  static_assert(!TAIL || C::HALVABLE, "tail tiles");
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_s = smem_u32(smem_raw);
   uint8_t* smem = smem_raw + ((1024u - (raw_s & 1023u)) & 1023u);
@@ -750,6 +783,9 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
     const uint32_t lead = elect_one() ? 1u : 0u;
     for (int i = 0; ok && i < nunits; ++i) {
       const Unit w = (!Sched::kMapsInGlobal && i == 0) ? first : sched.unit(i);
+      // a half unit loads its half of the tile's columns to the first half of the stage's B
+      const bool half = TAIL && w.half;
+      const int bx = w.tn * BN + (half ? w.noff * (BN / 2) : 0) + (P2 ? sched.rank * (half ? BN / 4 : BN / 2) : 0);
       for (int kb = w.kb0; kb < w.kb1; ++kb) {
         // a stage's first fill needs no wait: nothing has used it yet
         if (fills >= STAGES && !mbar_wait_warp(empty_bar(stage), ph ^ 1u, timeout, abort_flag)) {
@@ -760,12 +796,13 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
         const uint32_t sa = sbase + static_cast<uint32_t>(stage) * C::STAGE_BYTES;
         // pair: both CTAs' loads complete on the even CTA's full barrier, which expects both halves
         const uint32_t fb = P2 ? mapa_shared(full_bar(stage), 0) : full_bar(stage);
-        const int bx = w.tn * BN + (P2 ? sched.rank * (BN / 2) : 0);
-        mbar_arrive_expect_tx_lead(full_bar(stage), (P2 ? 2 : 1) * C::STAGE_BYTES, P2 && sched.rank != 0 ? 0u : lead);
+        mbar_arrive_expect_tx_lead(full_bar(stage), (P2 ? 2 : 1) * (C::STAGE_BYTES - (half ? C::B_BYTES / 2 : 0)),
+                                   P2 && sched.rank != 0 ? 0u : lead);
         tma_load_2d_lead<P2 ? 2 : 1>(sa, w.a, fb, kb * kBK, w.tm * BM, lead);
 #pragma unroll
         for (int j = 0; j < C::BN_LOAD / 64; ++j)
-          tma_load_2d_lead<P2 ? 2 : 1>(sa + C::A_BYTES + j * (kBK * 128), w.b, fb, bx + j * 64, kb * kBK, lead);
+          if (!half || j < C::BN_LOAD / 128)
+            tma_load_2d_lead<P2 ? 2 : 1>(sa + C::A_BYTES + j * (kBK * 128), w.b, fb, bx + j * 64, kb * kBK, lead);
         issued_mask |= 1u << stage;
         issued_ph = (issued_ph & ~(1u << stage)) | (ph << stage);
         if (++stage == STAGES) {
@@ -807,11 +844,13 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
     const int issue_units = (!P2 || sched.rank == 0) ? nunits : 0;
     // the K range and segments of the next unit, looked up while the current one's MMAs run
     int kb0n = 0, kb1n = 0, segsn = 1;
+    uint32_t idesc = C::IDESC;
     if (issue_units > 0) {
       const Unit w = sched.unit(0);
       kb0n = w.kb0;
       kb1n = w.kb1;
       segsn = w.segs;
+      if (TAIL && w.half) idesc = C::IDESC_HALF;
     }
     int seg = 0;
     for (int i = 0; ok && i < issue_units;) {
@@ -840,7 +879,7 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
 #pragma unroll
             for (int h = 0; h < C::HALVES; ++h)
               mma_f16_lead<P2 ? 2 : 1>(d0 + h * BN, alo0 + so + ((h * (128 * 128) + k * 32) >> 4), desc_hi,
-                                       blo0 + so + ((k * 2048) >> 4), desc_hi, C::IDESC, k > 0 ? 1u : first, lead);
+                                       blo0 + so + ((k * 2048) >> 4), desc_hi, idesc, k > 0 ? 1u : first, lead);
           }
           mma_commit_lead<P2 ? 2 : 1>(empty_bar(stage), lead);  // the stage is free (pair: in both CTAs)
         }
@@ -866,6 +905,7 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
         kb0n = w.kb0;
         kb1n = w.kb1;
         segsn = w.segs;
+        if (TAIL && w.half) idesc = C::IDESC_HALF;
       } else if (lane == 0) {
         RG_STAMP(5);
       }
@@ -1022,14 +1062,14 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
                         sbuf, lane);
         }
       } else if (!Sched::kSplit || w.splits == 1) {
+        const int cols = TAIL && w.half ? BN / 2 : BN, col0 = tn * BN + (TAIL && w.half ? w.noff * (BN / 2) : 0);
 #pragma unroll 1
         for (int h = 0; h < C::HALVES; ++h)
 #pragma unroll 1
-          for (int c = 0; c < BN / 32; ++c) {
+          for (int c = 0; c < cols / 32; ++c) {
             float v[32];
             load_acc(tacc + h * BN + c * 32, have, v);
-            store_block(w.c, v, tm * BM + h * 128 + q * 32, tn * BN + c * 32, w.M, w.N, w.beta, stg0, sbuf,
-                        lane);
+            store_block(w.c, v, tm * BM + h * 128 + q * 32, col0 + c * 32, w.M, w.N, w.beta, stg0, sbuf, lane);
           }
       } else if constexpr (Sched::kSplit) {
         // Split-K.  Publish this split's FP32 partial tile: TMEM -> swizzled staging ->
@@ -1265,8 +1305,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                      const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmW,
                      const GemmArgs args) {
-  SingleSched<SPLIT> sched{&tmA,        &tmB,          &tmC,   &tmW,  args.tiles_m, args.tiles_n,
-                           args.splits, args.kblocks, args.M, args.N, args.beta};
+  SingleSched<SPLIT, !SPLIT && KCfg<BM, BN, STAGES>::HALVABLE> sched{
+      &tmA, &tmB, &tmC, &tmW, args.tiles_m, args.tiles_n, args.splits, args.kblocks, args.M, args.N, args.beta};
+  sched.whole = args.whole;
   sched.panel = args.panel;
   gemm_body<BM, BN, STAGES>(sched, args.ws, args.tickets, args.err, args.timeout, args.stall, args.early, args.trace);
 }
@@ -1289,8 +1330,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     gemm_bf16_memtwin_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                              const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmW,
                              const GemmArgs args) {
-  MemTwinSched sched{{&tmA,        &tmB,          &tmC,   &tmW,  args.tiles_m, args.tiles_n,
-                      args.splits, args.kblocks, args.M, args.N, args.beta}};
+  MemTwinSched<KCfg<BM, BN, STAGES>::HALVABLE> sched{
+      {&tmA, &tmB, &tmC, &tmW, args.tiles_m, args.tiles_n, args.splits, args.kblocks, args.M, args.N, args.beta}};
+  sched.whole = args.whole;
   sched.panel = args.panel;
   gemm_body<BM, BN, STAGES>(sched, args.ws, args.tickets, args.err, args.timeout, args.stall, args.early, args.trace);
 }
@@ -1325,8 +1367,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     gemm_bf16_2sm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                          const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmW,
                          const GemmArgs args) {
-  TwoSmSched<SPLIT> sched{&tmA, &tmB, &tmC, &tmW, args.tiles_m, args.tiles_n, args.kblocks, args.M, args.N, args.beta};
+  TwoSmSched<SPLIT, !SPLIT && KCfg<128, BN, STAGES, 2>::HALVABLE> sched{
+      &tmA, &tmB, &tmC, &tmW, args.tiles_m, args.tiles_n, args.kblocks, args.M, args.N, args.beta};
   sched.splits = args.splits;
+  sched.whole = args.whole;
   sched.panel = args.panel;
   gemm_body<128, BN, STAGES>(sched, args.ws, args.tickets, args.err, args.timeout, args.stall, args.early, args.trace);
 }
@@ -1529,6 +1573,17 @@ static int make_map(CUtensorMap* m, CUtensorMapDataType dt, const void* base, ui
   return RG_OK;
 }
 
+// Tiles of the last, partial wave that run as two units of half the columns each: those r tiles of T = w P + r
+// (P CTAs, or clusters for pair tiles) for which the chip has room, w >= 1 and 2 r <= P; else 0.  The halves take
+// about half a tile's time (their MMAs have half the columns) on SMs that the last wave would leave idle; every
+// output is summed over K in the same order either way.  Tiles of 128 and 256 columns (pairs: 256).
+// 4096^3 on 256x256 pairs, r/P = 28/76: 80.1 -> 74.0 us; 4096 x 1280 x 4096, 4/76: 40.8 -> 32.6 (stream-K 40.4);
+// 2560 x 1024 x 2048 on 128x128, 8/152: 15.6 -> 13.7.
+static int64_t tail_tiles(int64_t tiles, int64_t p) {
+  const int64_t r = tiles % p;
+  return tiles >= p && 2 * r <= p ? r : 0;
+}
+
 struct Launch {
   KernFn fn = nullptr;
   CUtensorMap a, b, c, w;
@@ -1639,6 +1694,9 @@ static int prepare(rg_ctx* ctx, int64_t M, int64_t N, int64_t K, const void* A, 
   g.splits = sk ? static_cast<int32_t>(skg.tail_ctas) : splits;  // stream-K: CTAs sharing the tail tiles
   g.dp_tiles = sk ? static_cast<int32_t>(skg.dp_tiles) : 0;
   g.kblocks = static_cast<int32_t>(kblocks);
+  g.whole = static_cast<int32_t>(tiles_m * tiles_n);
+  if (splits == 1 && !sk && tk.bn % (two ? 256 : 128) == 0)
+    g.whole -= static_cast<int32_t>(tail_tiles(tiles_m * tiles_n, two ? ctx->sm_count / 2 : ctx->sm_count));
   {
     // column panels whose B slice (panel tiles x padded K, BF16) is at most 32 MiB
     const int64_t bcol = std::max<int64_t>(1, kblocks * kBK * tk.bn * 2);
