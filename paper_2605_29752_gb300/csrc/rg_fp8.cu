@@ -50,6 +50,7 @@
 #include <mutex>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "ptx.cuh"
@@ -145,6 +146,7 @@ struct Args {
   int32_t tiles_m, tiles_n;  // tiles of the (padded) launch
   int32_t kblocks;         // K blocks of the (padded) launch
   int32_t splits;
+  int32_t whole;           // tiles run whole, the rest as two half-width units each (see half_tiles)
   int32_t beta;
   int32_t mb_valid, kb_valid, nb_valid;  // logical scale blocks (reads beyond them are 0)
   int32_t sa_ld, sb_ld;    // leading dimensions of the scale arrays (blocks)
@@ -223,7 +225,17 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
   const int rank = PAIR ? static_cast<int>(cluster_ctarank()) : 0;
   const int cid = PAIR ? static_cast<int>(blockIdx.x) / 2 : static_cast<int>(blockIdx.x);
   const int ncl = PAIR ? static_cast<int>(gridDim.x) / 2 : static_cast<int>(gridDim.x);
-  const int total = (PAIR ? ntiles / 2 : ntiles) * S;
+  // Units: whole ones first, then (128 x 256 tile, S = 1) halves of the tiles from args.whole on, each
+  // one 128-column half of its tile's columns, promoted by the first four promotion warps; a CTA has at
+  // most one of them, its last.  Its loops are their own code, behind those of the whole units.
+  constexpr bool TAIL = C::HALVES == 2 && !SPLIT;
+  const int total = TAIL ? args.whole : (PAIR ? ntiles / 2 : ntiles) * S;
+  // the CTA's half unit (2 x its tile's place among the halved ones + the half), or -1
+  int half_unit = -1;
+  if constexpr (TAIL) {
+    const int h = (cid - total % ncl + ncl) % ncl;
+    if (h < 2 * (ntiles - args.whole)) half_unit = h;
+  }
   // unit u = ((pair) tile u / S, split u % S) runs K blocks [s * kblocks / S, (s + 1) * kblocks / S)
   auto kb_lo = [&](int s) { return S == 1 ? 0 : s * args.kblocks / S; };
   // this CTA's 128-row tile of unit u: tile index (tickets, workspace) and coordinates
@@ -281,26 +293,22 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
       uint32_t ph = 0, issued_mask = 0, issued_ph = 0;
       bool ok = true;
       const uint32_t lead = elect_one() ? 1u : 0u;
-      for (int u = cid; ok && u < total; u += ncl) {
-        const int s = u % S;
-        int tm, tn;
-        tile_of(u, tm, tn);
-        const int kb1 = s + 1 == S ? args.kblocks : kb_lo(s + 1);
-        for (int kb = kb_lo(s); kb < kb1; ++kb) {
+      // loads K blocks [kb0, kb1) of tile (tm, tn): all of its columns, or (a half) one box from column bx
+      auto load = [&](int tm, int bx, int kb0, int kb1, auto boxes) {
+        constexpr int kBoxes = decltype(boxes)::value;
+        for (int kb = kb0; kb < kb1; ++kb) {
           if (fills >= C::STAGES &&
-              !mbar_wait_warp(COUPLED ? tempty_bar(stage) : empty_bar(stage), ph ^ 1u, args.timeout, abort_flag)) {
-            ok = false;
-            break;
-          }
+              !mbar_wait_warp(COUPLED ? tempty_bar(stage) : empty_bar(stage), ph ^ 1u, args.timeout, abort_flag))
+            return false;
           ++fills;
           const uint32_t sa = sbase + static_cast<uint32_t>(stage) * C::STAGE_BYTES;
           // pair: both CTAs' loads complete on the even CTA's full barrier, which expects both halves
           const uint32_t fb = PAIR ? mapa_shared(full_bar(stage), 0) : full_bar(stage);
-          const int bx = tn * BN + (PAIR ? rank * (BN / 2) : 0);
-          mbar_arrive_expect_tx_lead(full_bar(stage), C::CTAS * C::STAGE_BYTES, PAIR && rank != 0 ? 0u : lead);
+          mbar_arrive_expect_tx_lead(full_bar(stage), C::CTAS * (C::A_BYTES + kBoxes * BK * 128),
+                                     PAIR && rank != 0 ? 0u : lead);
           tma_load_2d_lead<C::CTAS>(sa, &tmA, fb, kb * BK, tm * BM, lead);
 #pragma unroll
-          for (int j = 0; j < BN / C::CTAS / 128; ++j)
+          for (int j = 0; j < kBoxes; ++j)
             tma_load_2d_lead<C::CTAS>(sa + C::A_BYTES + j * (BK * 128), &tmB, fb, bx + j * 128, kb * BK, lead);
           issued_mask |= 1u << stage;
           issued_ph = (issued_ph & ~(1u << stage)) | (ph << stage);
@@ -308,6 +316,21 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
             stage = 0;
             ph ^= 1u;
           }
+        }
+        return true;
+      };
+      for (int u = cid; ok && u < total; u += ncl) {
+        const int s = u % S;
+        int tm, tn;
+        tile_of(u, tm, tn);
+        ok = load(tm, tn * BN + (PAIR ? rank * (BN / 2) : 0), kb_lo(s), s + 1 == S ? args.kblocks : kb_lo(s + 1),
+                  std::integral_constant<int, BN / C::CTAS / 128>{});
+      }
+      if constexpr (TAIL) {
+        if (ok && half_unit >= 0) {
+          int tm, tn;
+          tile_of(args.whole + half_unit / 2, tm, tn);
+          ok = load(tm, tn * BN + half_unit % 2 * 128, 0, args.kblocks, std::integral_constant<int, 1>{});
         }
       }
       if (lane == 0) {
@@ -340,19 +363,16 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
         const uint64_t bdesc0 = smem_desc_sw128(sbase + C::A_BYTES, BK * 128, 1024);  // column boxes BK*128 apart
         const uint32_t alo0 = static_cast<uint32_t>(adesc0), blo0 = static_cast<uint32_t>(bdesc0);
         const uint32_t desc_hi = static_cast<uint32_t>(adesc0 >> 32);  // that of both: same stride and swizzle
-        for (int u = cid; ok && u < total; u += ncl) {
-          const int s = u % S;
-          const int kb1 = s + 1 == S ? args.kblocks : kb_lo(s + 1);
-          for (int kb = kb_lo(s); kb < kb1; ++kb) {
-            ok = mbar_wait_warp(full_bar(stage), ph, args.timeout, abort_flag);
-            if (!ok) break;
+        // the MMAs of n K blocks, the first `halves` column halves of each
+        auto multiply = [&](int n, auto halves) {
+          for (int i = 0; i < n; ++i) {
+            if (!mbar_wait_warp(full_bar(stage), ph, args.timeout, abort_flag)) return false;
             const uint32_t so = static_cast<uint32_t>(stage) * (C::STAGE_BYTES >> 4);
 #pragma unroll
-            for (int h = 0; h < C::HALVES; ++h) {
+            for (int h = 0; h < decltype(halves)::value; ++h) {
               const int buf = acc * C::HALVES + h;
               if constexpr (!COUPLED) {
-                if (ok) ok = mbar_wait_warp(tempty_bar(buf), aph ^ 1u, args.timeout, abort_flag);
-                if (!ok) break;
+                if (!mbar_wait_warp(tempty_bar(buf), aph ^ 1u, args.timeout, abort_flag)) return false;
               }
               tc_fence_after();
               constexpr uint32_t hb = (BK * 128) >> 4;  // half h of the B columns is the h-th column box
@@ -363,7 +383,6 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
                                      lead);
               mma_commit_lead<C::CTAS>(tfull_bar(buf), lead);  // pair: both CTAs' rows of the product are ready
             }
-            if (!ok) break;
             if (++stage == C::STAGES) {
               stage = 0;
               ph ^= 1u;
@@ -373,6 +392,14 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
               aph ^= 1u;
             }
           }
+          return true;
+        };
+        for (int u = cid; ok && u < total; u += ncl) {
+          const int s = u % S;
+          ok = multiply((s + 1 == S ? args.kblocks : kb_lo(s + 1)) - kb_lo(s), std::integral_constant<int, C::HALVES>{});
+        }
+        if constexpr (TAIL) {
+          if (ok && half_unit >= 0) ok = multiply(args.kblocks, std::integral_constant<int, 1>{});
         }
         if (!ok) {
           if (elect_one()) {
@@ -399,23 +426,20 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
     int acc = 0, sbuf = 0, pstage = 0;  // pstage: the operand stage of the current K block
     uint32_t aph = 0;
     bool ok = true;
-    for (int u = cid; ok && u < total; u += ncl) {
-      const int s = u % S;
-      int tm, tn;
-      const int tile = tile_of(u, tm, tn);
-      const int kb1 = s + 1 == S ? args.kblocks : kb_lo(s + 1);
-      const int nb = (tn * BN + hc * C::HALF) / SB;  // this half's scale block column
+    // promotes K blocks [kb0, kb1) of the tile's row block tm and the warp's columns from `col` on into r;
+    // half: of a half unit, whose one buffer per K block the first four warps read
+    auto promote = [&](int tm, int col, int kb0, int kb1, float (&r)[C::HALF], auto half) {
+      const int nb = col / SB;  // the scale block column
       // scale rows and the last K block with real scales (0 outside the logical blocks: padding)
       const int kbv = (tm < args.mb_valid && nb < args.nb_valid) ? args.kb_valid : 0;
-      float r[C::HALF];
 #pragma unroll
       for (int i = 0; i < C::HALF; ++i) r[i] = 0.f;
       // The K blocks' scale products, 32 at a time, one per lane: lane l holds that of K block
       // kb0 + 32 j + l.  A load per K block would put its global-memory latency on the promotion's
       // critical path whenever the block's product is already waiting in TMEM.
       float sc_lane = 0.f;
-      for (int kb = kb_lo(s); kb < kb1; ++kb) {
-        const int rel = kb - kb_lo(s);
+      for (int kb = kb0; kb < kb1; ++kb) {
+        const int rel = kb - kb0;
         if ((rel & 31) == 0) {
           // (scale pointers are recomputed from the kernel parameters: registers are scarce here)
           const int k = kb + lane;
@@ -425,10 +449,9 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
         }
         const float sc = __shfl_sync(FULL, sc_lane, rel & 31);
         const int buf = C::HALVES == 2 ? 2 * acc + hc : acc;
-        ok = mbar_wait_warp(tfull_bar(buf), aph, args.timeout, abort_flag);
-        if (!ok) break;
+        if (!mbar_wait_warp(tfull_bar(buf), aph, args.timeout, abort_flag)) return false;
         if constexpr (!COUPLED) {
-          if (e == (C::HALVES - 1) * 4 && lane == 0) mbar_arrive(empty_bar(pstage));  // this CTA's copy of the stage is free
+          if (e == (decltype(half)::value ? 0 : (C::HALVES - 1) * 4) && lane == 0) mbar_arrive(empty_bar(pstage));  // this CTA's copy of the stage is free
           if (++pstage == C::STAGES) pstage = 0;
         }
         tc_fence_after();
@@ -462,6 +485,14 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
           aph ^= 1u;
         }
       }
+      return true;
+    };
+    for (int u = cid; ok && u < total; u += ncl) {
+      const int s = u % S;
+      int tm, tn;
+      const int tile = tile_of(u, tm, tn);
+      float r[C::HALF];
+      ok = promote(tm, tn * BN + hc * C::HALF, kb_lo(s), s + 1 == S ? args.kblocks : kb_lo(s + 1), r, std::false_type{});
       if (!ok) break;
       const int row0 = tm * BM + q * 32;
       if constexpr (!SPLIT) {
@@ -529,6 +560,20 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
         const int col0 = tn * BN + hc * C::HALF + c * 32;
         if (row0 < args.M && col0 < args.N) put_block<C::NSTG>(&tmC, sum, row0, col0, args.beta != 0, stg0, sbuf, lane);
       }
+      }
+    }
+    if constexpr (TAIL) {
+      if (ok && half_unit >= 0 && hc == 0) {
+        int tm, tn;
+        tile_of(args.whole + half_unit / 2, tm, tn);
+        const int col = tn * BN + half_unit % 2 * C::HALF;
+        float r[C::HALF];
+        ok = promote(tm, col, 0, args.kblocks, r, std::true_type{});
+        if (ok)
+#pragma unroll
+          for (int c = 0; c < C::HALF / 32; ++c)
+            if (tm * BM + q * 32 < args.M && col + c * 32 < args.N)
+              put_block<C::NSTG>(&tmC, r + c * 32, tm * BM + q * 32, col + c * 32, args.beta != 0, stg0, sbuf, lane);
       }
     }
     if (!ok && lane == 0) {
@@ -740,6 +785,14 @@ struct Launch {
   int64_t M = 0, N = 0, ldc = 0;
 };
 
+// 128 x 256 tiles of the last (or only) wave that run as two units of half the columns each: those r = T mod P of
+// T tiles on P SMs where 2 r <= P, so that the halves fill SMs the wave would leave idle.  A half takes about 0.65
+// of a tile's time, and every output is summed over K in the same order.  FP8_TAIL
+static int64_t half_tiles(int64_t tiles, int64_t p) {
+  const int64_t r = tiles % p;
+  return 2 * r <= p ? r : 0;
+}
+
 // Checks one FP8 GEMM launch and builds its tensor maps and arguments.
 static int prepare(const Fp8CtxInfo& info, int64_t M, int64_t N, int64_t K, const uint8_t* qA, int64_t lda,
                    const float* sA, int64_t lds_a, const uint8_t* qB, int64_t ldb, const float* sB, int64_t lds_b,
@@ -783,6 +836,7 @@ static int prepare(const Fp8CtxInfo& info, int64_t M, int64_t N, int64_t K, cons
   if (ti.pair) tiles_m += tiles_m & 1;  // whole 256-row pair tiles (an odd CTA past M loads zeros, stores nothing)
   const int64_t tiles_n = (pn + ti.bn - 1) / ti.bn, kblocks = (pk + BK - 1) / BK;
   const int64_t ntiles = tiles_m * tiles_n;
+  const int64_t halves = ti.pair || ti.bn != 256 || splits > 1 ? 0 : half_tiles(ntiles, info.sms);
   if (splits > 1 && (splits * ntiles * BM * ti.bn * 4 > info.ws_bytes || ntiles * kEpiWarps > info.max_tickets))
     return fail(RG_ERR_SHAPE, "FP8 GEMM: split-K workspace too small for this shape");
   if (ntiles * splits > (1LL << 30)) return fail(RG_ERR_SHAPE, "FP8 GEMM: too many work units");
@@ -804,6 +858,7 @@ static int prepare(const Fp8CtxInfo& info, int64_t M, int64_t N, int64_t K, cons
   g.tiles_n = static_cast<int32_t>(tiles_n);
   g.kblocks = static_cast<int32_t>(kblocks);
   g.splits = splits;
+  g.whole = static_cast<int32_t>(ntiles - halves);
   g.beta = beta;
   g.mb_valid = static_cast<int32_t>(mb_valid);
   g.kb_valid = static_cast<int32_t>(kb_valid);
@@ -819,7 +874,7 @@ static int prepare(const Fp8CtxInfo& info, int64_t M, int64_t N, int64_t K, cons
   L->fn = splits > 1 ? ti.fn_split : ti.fn;
   L->smem = ti.smem;
   L->grid = ti.pair ? dim3(static_cast<unsigned>(2 * std::min<int64_t>(ntiles / 2 * splits, info.sms / 2)))
-                    : dim3(static_cast<unsigned>(std::min<int64_t>(ntiles * splits, info.sms)));
+                    : dim3(static_cast<unsigned>(std::min<int64_t>(ntiles * splits + halves, info.sms)));
   return RG_OK;
 }
 
