@@ -1423,6 +1423,32 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   gemm_body<128, BN, STAGES>(sched, ws, tickets, err, timeout, 0, 0);
 }
 
+// Rows of a pinned host matrix to device memory, as elements of type V (the widest its addresses and pitches
+// allow: 16, 4 or 2 bytes).  Bound by the host link, which the SMs' loads fill as a copy engine's do (16.8 MB:
+// 203 GB/s by a copy engine, 196 by 16-byte and 189 by 2-byte loads) -- but a copy engine takes rows that do not
+// start on a vector boundary at 72 GB/s.  128 threads to a matrix row, kCopyBatch loads of each
+// thread in flight; enough CTAs to fill the link with 2-byte loads, and small enough to sit beside a GEMM's.
+constexpr int kRowCtas = 304, kRowThreads = 128, kRowRows = 4, kCopyBatch = 8;
+template <class V>
+__global__ void __launch_bounds__(kRowThreads* kRowRows)
+    copy_rows_kernel(const unsigned char* __restrict__ src, int64_t src_pitch, unsigned char* __restrict__ dst,
+                     int64_t dst_pitch, int64_t row_items, int64_t rows) {
+  for (int64_t r = static_cast<int64_t>(blockIdx.x) * kRowRows + threadIdx.y; r < rows;
+       r += static_cast<int64_t>(gridDim.x) * kRowRows) {
+    const V* s = reinterpret_cast<const V*>(src + r * src_pitch);
+    V* d = reinterpret_cast<V*>(dst + r * dst_pitch);
+    int64_t i = threadIdx.x;
+    for (; i + (kCopyBatch - 1) * kRowThreads < row_items; i += kCopyBatch * kRowThreads) {
+      V v[kCopyBatch];
+#pragma unroll
+      for (int j = 0; j < kCopyBatch; ++j) v[j] = s[i + j * kRowThreads];
+#pragma unroll
+      for (int j = 0; j < kCopyBatch; ++j) d[i + j * kRowThreads] = v[j];
+    }
+    for (; i < row_items; i += kRowThreads) d[i] = s[i];
+  }
+}
+
 // Device-side spin of about `ns` nanoseconds (global timer), so that launches
 // enqueued behind it start back to back.  Bounded by a cycle cap as well.
 __global__ void spin_kernel(long long ns) {
@@ -2101,6 +2127,43 @@ int grow_stage(void** buf, int64_t* cap, int64_t bytes, cudaStream_t st) {
   *cap = bytes;
   return RG_OK;
 }
+
+// Whether the device can read [p, p + bytes) itself: page-locked host memory at its own address.
+bool pinned(const void* p, int64_t bytes) {
+  const auto* c = static_cast<const unsigned char*>(p);
+  for (const unsigned char* at : {c, c + bytes - 1}) {
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, at) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (a.type != cudaMemoryTypeHost || a.devicePointer != at) return false;
+  }
+  return true;
+}
+
+// Rows of a host matrix to a staging buffer (16-byte aligned, its pitch a multiple of 16): by a copy engine where
+// they are one block of memory or pageable, else by the SMs (8.4 MB in rows of 4,090
+// bytes: 117 us by a copy engine, 47 so; whole calls of 2047^3 361 -> 237 us, 1001 x 1095 x 1303 182 -> 97).
+cudaError_t rows_in(void* dst, int64_t dst_pitch, const void* src, int64_t src_pitch, int64_t row_bytes, int64_t rows,
+                    cudaStream_t st) {
+  const uintptr_t at = reinterpret_cast<uintptr_t>(src);
+  const bool block = rows == 1 || (src_pitch == row_bytes && dst_pitch == row_bytes);
+  if (block || at % 2 != 0 || !pinned(src, (rows - 1) * src_pitch + row_bytes))
+    return cudaMemcpy2DAsync(dst, dst_pitch, src, src_pitch, row_bytes, rows, cudaMemcpyHostToDevice, st);
+  const uintptr_t bits = at | static_cast<uintptr_t>(src_pitch) | static_cast<uintptr_t>(row_bytes);
+  const dim3 grid(static_cast<unsigned>(std::min<int64_t>((rows + rg::kRowRows - 1) / rg::kRowRows, rg::kRowCtas)));
+  const dim3 block_dim(rg::kRowThreads, rg::kRowRows);
+  const auto* s = static_cast<const unsigned char*>(src);
+  auto* d = static_cast<unsigned char*>(dst);
+  if (bits % 16 == 0)
+    rg::copy_rows_kernel<uint4><<<grid, block_dim, 0, st>>>(s, src_pitch, d, dst_pitch, row_bytes / 16, rows);
+  else if (bits % 4 == 0)
+    rg::copy_rows_kernel<uint32_t><<<grid, block_dim, 0, st>>>(s, src_pitch, d, dst_pitch, row_bytes / 4, rows);
+  else
+    rg::copy_rows_kernel<uint16_t><<<grid, block_dim, 0, st>>>(s, src_pitch, d, dst_pitch, row_bytes / 2, rows);
+  return cudaGetLastError();
+}
 }  // namespace
 
 extern "C" int rg_gemm_plan_host(rg_ctx* ctx, const rg_plan* plan, int64_t M, int64_t N, int64_t K, const void* A,
@@ -2118,12 +2181,16 @@ extern "C" int rg_gemm_plan_host(rg_ctx* ctx, const rg_plan* plan, int64_t M, in
   if (rc == RG_OK)
     rc = grow_stage(reinterpret_cast<void**>(&ctx->stage_c), &ctx->stage_c_bytes, 4 * M * dldc, st);
   if (rc != RG_OK) return rc;
-  cudaError_t e = cudaMemcpy2DAsync(ctx->stage_a, dlda * 2, A, lda * 2, K * 2, M, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess)
-    e = cudaMemcpy2DAsync(ctx->stage_b, dldb * 2, B, ldb * 2, N * 2, K, cudaMemcpyHostToDevice, st);
+  cudaError_t e = rows_in(ctx->stage_a, dlda * 2, A, lda * 2, K * 2, M, st);
+  if (e == cudaSuccess) e = rows_in(ctx->stage_b, dldb * 2, B, ldb * 2, N * 2, K, st);
   if (e != cudaSuccess) return rg::cuda_fail(e, "rg_gemm_plan_host: copy in");
-  rc = rg_gemm_plan(ctx, plan, M, N, K, ctx->stage_a, dlda, ctx->stage_b, dldb, ctx->stage_c, dldc, stream);
+  std::vector<rg::Launch> ls;
+  rc = rg::plan_launches(ctx, plan, M, N, K, ctx->stage_a, dlda, ctx->stage_b, dldb, ctx->stage_c, dldc, ls);
   if (rc != RG_OK) return rc;
+  for (auto& L : ls) {
+    L.args.early = 0;  // the staged operands are the copies' results, whatever the caller's own operands are
+    if ((e = rg::launch(ctx, L, st)) != cudaSuccess) return rg::cuda_fail(e, "rg_gemm_plan_host: launch");
+  }
   e = cudaMemcpy2DAsync(C, ldc * 4, ctx->stage_c, dldc * 4, N * 4, M, cudaMemcpyDeviceToHost, st);
   if (e != cudaSuccess) return rg::cuda_fail(e, "rg_gemm_plan_host: copy out");
   return rg_check(ctx, stream);
