@@ -1537,6 +1537,8 @@ static int family_of(int v) {
   return variant_2sm(v) ? RG_NUM_TILES + RG_PAIR_INDEX(variant_tile(v)) : variant_tile(v);
 }
 
+constexpr int kMaxPanels = 4;  // rg_gemm_plan_host: row panels of an overlapped call
+
 }  // namespace rg
 
 struct rg_ctx {
@@ -1559,6 +1561,9 @@ struct rg_ctx {
   void* stage_b = nullptr;
   float* stage_c = nullptr;
   int64_t stage_a_bytes = 0, stage_b_bytes = 0, stage_c_bytes = 0;
+  // its copies beside the GEMMs (made on first use): the caller's earlier work, the last copy out, panels in, computed
+  cudaStream_t copy_in = nullptr, copy_out = nullptr;
+  cudaEvent_t host_ev[2 + 2 * rg::kMaxPanels] = {};
 };
 
 namespace rg {
@@ -1620,6 +1625,7 @@ struct Launch {
   bool noop = false;
   int64_t ws_slots = 1;  // > 1: the launch uses the split-K workspace and tickets
   int cluster = 1;       // 2: launched as 2-CTA clusters
+  bool streamk = false;
   float* C = nullptr;
   int64_t M = 0, N = 0, ldc = 0;
 };
@@ -1712,6 +1718,7 @@ static int prepare(rg_ctx* ctx, int64_t M, int64_t N, int64_t K, const void* A, 
   L->cluster = two ? 2 : csplit ? splits : 1;
   L->smem = two ? tk.smem2 : tk.smem;
   L->ws_slots = slots;
+  L->streamk = sk;
   GemmArgs& g = L->args;
   g.M = static_cast<int32_t>(M);
   g.N = static_cast<int32_t>(N);
@@ -1785,9 +1792,11 @@ void ctx_identity(const rg_ctx* ctx, char name[64], int32_t* sms) {
   *sms = ctx->sm_count;
 }
 
-// Leaves of the plan cell covering (M, N, K), clipped to the problem.
+// Leaves of the plan cell covering (M, N, K), clipped to the problem and to its rows [row0, row1) (where they keep
+// their padded K, and so the sums of the whole problem; padded rows change no sum).
 static int plan_launches(rg_ctx* ctx, const rg_plan* plan, int64_t M, int64_t N, int64_t K, const void* A,
-                         int64_t lda, const void* B, int64_t ldb, float* C, int64_t ldc, std::vector<Launch>& out) {
+                         int64_t lda, const void* B, int64_t ldb, float* C, int64_t ldc, std::vector<Launch>& out,
+                         int64_t row0 = 0, int64_t row1 = INT64_MAX) {
   out.clear();
   if (!plan) return fail(RG_ERR_INVALID, "null plan");
   if (M <= 0 || N <= 0 || K <= 0) return fail(RG_ERR_INVALID, "plan execution needs positive sizes");
@@ -1799,12 +1808,20 @@ static int plan_launches(rg_ctx* ctx, const rg_plan* plan, int64_t M, int64_t N,
   for (int64_t i = P.leaf_off[cell]; i < P.leaf_off[cell + 1]; ++i) {
     const rg_leaf& lf = P.leaves[i];
     if (lf.m0 >= M || lf.n0 >= N || lf.k0 >= K) continue;  // wholly in the padding
-    const int64_t m = std::min(lf.m, M - lf.m0), n = std::min(lf.n, N - lf.n0), k = std::min(lf.k, K - lf.k0);
-    const auto* a = static_cast<const uint16_t*>(A) + lf.m0 * lda + lf.k0;
+    int64_t m0 = lf.m0, m = std::min(lf.m, M - m0), pm = lf.pm;
+    const int64_t n = std::min(lf.n, N - lf.n0), k = std::min(lf.k, K - lf.k0);
+    if (m0 < row0 || m0 + m > row1) {
+      const int64_t end = std::min(m0 + m, row1);
+      m0 = std::max(m0, row0);
+      m = end - m0;
+      pm = 0;
+      if (m <= 0) continue;
+    }
+    const auto* a = static_cast<const uint16_t*>(A) + m0 * lda + lf.k0;
     const auto* b = static_cast<const uint16_t*>(B) + lf.k0 * ldb + lf.n0;
-    float* c = C + lf.m0 * ldc + lf.n0;
+    float* c = C + m0 * ldc + lf.n0;
     Launch L;
-    const int rc = prepare(ctx, m, n, k, a, lda, b, ldb, c, ldc, lf.variant, lf.beta, lf.pm, lf.pn, lf.pk, &L);
+    const int rc = prepare(ctx, m, n, k, a, lda, b, ldb, c, ldc, lf.variant, lf.beta, pm, lf.pn, lf.pk, &L);
     if (rc != RG_OK) return rc;
     out.push_back(L);
   }
@@ -1993,6 +2010,10 @@ extern "C" void rg_destroy(rg_ctx* ctx) {
   if (!ctx) return;
   cudaSetDevice(ctx->device);
   for (auto ev : ctx->events) cudaEventDestroy(ev);
+  for (auto ev : ctx->host_ev)
+    if (ev) cudaEventDestroy(ev);
+  if (ctx->copy_in) cudaStreamDestroy(ctx->copy_in);
+  if (ctx->copy_out) cudaStreamDestroy(ctx->copy_out);
   cudaFree(ctx->trace);
   cudaFree(ctx->stage_a);
   cudaFree(ctx->stage_b);
@@ -2164,6 +2185,68 @@ cudaError_t rows_in(void* dst, int64_t dst_pitch, const void* src, int64_t src_p
     rg::copy_rows_kernel<uint16_t><<<grid, block_dim, 0, st>>>(s, src_pitch, d, dst_pitch, row_bytes / 2, rows);
   return cudaGetLastError();
 }
+
+// Row panels of an overlapped call.  The host link carries both directions at once (16.8 MB each way: 83 + 95 us in
+// turn, 110 together), so C's panels go back while A's later ones come in and are multiplied.  A panel is at least
+// 40 us of C's way out (shorter ones lose to their copies' and launches' own time), whole 256-row tiles, and its GEMM,
+// at least one tile's time (K blocks x 0.26 us + 4), no longer than its way out.  2048^3: 214 us whole, 198 in two
+// panels, 204 in four; 3072^3: 444, 402 and 381.
+int choose_panels(int64_t M, int64_t N, int64_t K) {
+  const double out_us = 4.0 * M * N / 177e3, gemm_us = (K + 63) / 64 * 0.26 + 4.0;
+  const double n = std::min(out_us / std::max(40.0, gemm_us), M / 256.0);
+  return n < 2 ? 1 : n < rg::kMaxPanels ? static_cast<int>(n) : rg::kMaxPanels;
+}
+
+// The call in panels: operands come in on one stream, panels are computed on the caller's and go out on a third, all of
+// it joined to `st`.  A and B are one block of memory each.
+int host_panels(rg_ctx* ctx, const rg_plan* plan, int panels, int64_t M, int64_t N, int64_t K, const void* A,
+                const void* B, float* C, int64_t ldc, int64_t dldc, cudaStream_t st) {
+  cudaError_t e = cudaSuccess;
+  if (!ctx->copy_in) e = cudaStreamCreateWithFlags(&ctx->copy_in, cudaStreamNonBlocking);
+  if (e == cudaSuccess && !ctx->copy_out) e = cudaStreamCreateWithFlags(&ctx->copy_out, cudaStreamNonBlocking);
+  for (auto& ev : ctx->host_ev)
+    if (e == cudaSuccess && !ev) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+  cudaEvent_t *in = ctx->host_ev + 2, *done = in + rg::kMaxPanels;
+  auto end_row = [&](int i) { return i + 1 == panels ? M : M * (i + 1) / panels / 256 * 256; };
+  if (e == cudaSuccess) e = cudaEventRecord(ctx->host_ev[0], st);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->copy_in, ctx->host_ev[0], 0);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->stage_b, B, 2 * K * N, cudaMemcpyHostToDevice, ctx->copy_in);
+  for (int i = 0; i < panels && e == cudaSuccess; ++i) {
+    const int64_t at = i ? 2 * K * end_row(i - 1) : 0;
+    e = cudaMemcpyAsync(static_cast<unsigned char*>(ctx->stage_a) + at, static_cast<const unsigned char*>(A) + at,
+                        2 * K * end_row(i) - at, cudaMemcpyHostToDevice, ctx->copy_in);
+    if (e == cudaSuccess) e = cudaEventRecord(in[i], ctx->copy_in);
+  }
+  int rc = RG_OK;
+  std::vector<rg::Launch> ls;
+  for (int i = 0; i < panels && e == cudaSuccess && rc == RG_OK; ++i) {
+    const int64_t row0 = i ? end_row(i - 1) : 0, row1 = end_row(i);
+    rc = rg::plan_launches(ctx, plan, M, N, K, ctx->stage_a, K, ctx->stage_b, N, ctx->stage_c, dldc, ls, row0, row1);
+    if (rc != RG_OK) break;
+    e = cudaStreamWaitEvent(st, in[i], 0);
+    for (size_t l = 0; e == cudaSuccess && l < ls.size(); ++l) {
+      ls[l].args.early = 0;
+      e = rg::launch(ctx, ls[l], st);
+    }
+    if (e == cudaSuccess) e = cudaEventRecord(done[i], st);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->copy_out, done[i], 0);
+    if (e == cudaSuccess)
+      e = cudaMemcpy2DAsync(C + row0 * ldc, ldc * 4, ctx->stage_c + row0 * dldc, dldc * 4, N * 4, row1 - row0,
+                            cudaMemcpyDeviceToHost, ctx->copy_out);
+  }
+  if (e == cudaSuccess && rc == RG_OK) e = cudaEventRecord(ctx->host_ev[1], ctx->copy_out);
+  if (e == cudaSuccess && rc == RG_OK) e = cudaStreamWaitEvent(st, ctx->host_ev[1], 0);
+  if (e == cudaSuccess && rc == RG_OK) return RG_OK;
+  // after an error nothing may still touch the caller's buffers
+  if (ctx->copy_in) cudaStreamSynchronize(ctx->copy_in);
+  if (ctx->copy_out) cudaStreamSynchronize(ctx->copy_out);
+  return rc != RG_OK ? rc : rg::cuda_fail(e, "rg_gemm_plan_host: panels");
+}
+
+bool overlap(const void* a, int64_t na, const void* b, int64_t nb) {
+  const auto x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+  return x < y + static_cast<uintptr_t>(nb) && y < x + static_cast<uintptr_t>(na);
+}
 }  // namespace
 
 extern "C" int rg_gemm_plan_host(rg_ctx* ctx, const rg_plan* plan, int64_t M, int64_t N, int64_t K, const void* A,
@@ -2181,12 +2264,25 @@ extern "C" int rg_gemm_plan_host(rg_ctx* ctx, const rg_plan* plan, int64_t M, in
   if (rc == RG_OK)
     rc = grow_stage(reinterpret_cast<void**>(&ctx->stage_c), &ctx->stage_c_bytes, 4 * M * dldc, st);
   if (rc != RG_OK) return rc;
-  cudaError_t e = rows_in(ctx->stage_a, dlda * 2, A, lda * 2, K * 2, M, st);
-  if (e == cudaSuccess) e = rows_in(ctx->stage_b, dldb * 2, B, ldb * 2, N * 2, K, st);
-  if (e != cudaSuccess) return rg::cuda_fail(e, "rg_gemm_plan_host: copy in");
   std::vector<rg::Launch> ls;
   rc = rg::plan_launches(ctx, plan, M, N, K, ctx->stage_a, dlda, ctx->stage_b, dldb, ctx->stage_c, dldc, ls);
   if (rc != RG_OK) return rc;
+  // In panels where the copies are plain ones and can run beside each other: A and B one block of memory each, all
+  // three buffers page-locked, C apart from A and B, and no stream-K leaf (which tiles share sums there depends on
+  // how many there are).  (With rows copied by the SMs, 1001 x 1095 x 1303 took 114 us in panels, 98 whole.)
+  const int panels = lda == K && dlda == K && ldb == N && dldb == N ? choose_panels(M, N, K) : 1;
+  if (panels > 1) {
+    const int64_t na = 2 * M * K, nb = 2 * K * N, nc = 4 * ((M - 1) * ldc + N);
+    bool apart = !overlap(A, na, C, nc) && !overlap(B, nb, C, nc) && pinned(A, na) && pinned(B, nb) && pinned(C, nc);
+    for (const auto& L : ls) apart = apart && !L.streamk;
+    if (apart) {
+      rc = host_panels(ctx, plan, panels, M, N, K, A, B, C, ldc, dldc, st);
+      return rc == RG_OK ? rg_check(ctx, stream) : rc;
+    }
+  }
+  cudaError_t e = rows_in(ctx->stage_a, dlda * 2, A, lda * 2, K * 2, M, st);
+  if (e == cudaSuccess) e = rows_in(ctx->stage_b, dldb * 2, B, ldb * 2, N * 2, K, st);
+  if (e != cudaSuccess) return rg::cuda_fail(e, "rg_gemm_plan_host: copy in");
   for (auto& L : ls) {
     L.args.early = 0;  // the staged operands are the copies' results, whatever the caller's own operands are
     if ((e = rg::launch(ctx, L, st)) != cudaSuccess) return rg::cuda_fail(e, "rg_gemm_plan_host: launch");
