@@ -105,6 +105,7 @@ struct GemmArgs {
   int32_t dp_tiles;         // stream-K: tiles run whole before the shared tail
   int32_t panel;            // tile order: column panels of this many tiles (pairs: tile columns)
   int32_t early;            // 1: A and B are static, so loads may start before the preceding grid completes
+  int32_t segs;             // accumulators a unit's K blocks are summed in, one after another (see accum_segs)
   int32_t whole;            // (pair) tiles run whole, the rest as two half-width units each (see tail_tiles)
   float* ws;                // split-K partials [split][tile][BM][BN]
   int32_t* tickets;         // [tile][4], zero between launches
@@ -217,6 +218,8 @@ __device__ __forceinline__ void store_block(const CUtensorMap* tmC, const float 
 // Whether a tile's grouped units may run all K splits of a problem in turn: its epilogue threads
 // then hold one FP32 sum per accumulator column (TMEM columns: BN, twice that for 256-row CTAs).
 __host__ __device__ constexpr bool serial_tile(int acc_cols) { return acc_cols <= 128; }
+// Whether its units may sum their K blocks in several accumulators in turn (1-CTA tiles).
+__host__ __device__ constexpr bool segment_tile(int acc_cols) { return acc_cols <= 192; }
 
 // One work unit: which output tile of which problem, which K blocks, and where
 // its operands and output live.
@@ -296,6 +299,7 @@ struct SingleSched {
   const CUtensorMap* w;
   int tiles_m, tiles_n, splits, kblocks, M, N, beta;
   int whole = 0;
+  int segs = 1;
   int panel = 1 << 30;
   __device__ __forceinline__ void prefetch() const {
     prefetch_tmap(a);
@@ -318,6 +322,7 @@ struct SingleSched {
       x.half = u >= whole;
       x.noff = h & 1;
     }
+    if constexpr (!SPLIT) x.segs = segs;
     return x;
   }
 };
@@ -687,7 +692,8 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
   constexpr bool CS = IsClusterSplit<Sched>::value;  // one K slice of a cluster split-K tile
   using C = KCfg<BM, BN, STAGES, P2 ? 2 : 1>;
   // units may run all K splits of their tile (a thread then holds its sums of the whole tile in registers)
-  constexpr bool SERIAL = Sched::kMapsInGlobal && serial_tile(C::ACC_COLS);
+  constexpr bool SERIAL = Sched::kMapsInGlobal ? (P2 ? serial_tile(C::ACC_COLS) : segment_tile(C::ACC_COLS))
+                                               : !Sched::kSplit && !CS && !P2 && !Sched::kMemOnly && segment_tile(C::ACC_COLS);
   constexpr bool TAIL = HasTail<Sched>::value;  // units may be halves of their tile's columns
   static_assert(!TAIL || C::HALVABLE, "tail tiles");
   extern __shared__ uint8_t smem_raw[];
@@ -1308,6 +1314,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   SingleSched<SPLIT, !SPLIT && KCfg<BM, BN, STAGES>::HALVABLE> sched{
       &tmA, &tmB, &tmC, &tmW, args.tiles_m, args.tiles_n, args.splits, args.kblocks, args.M, args.N, args.beta};
   sched.whole = args.whole;
+  sched.segs = args.segs;
   sched.panel = args.panel;
   gemm_body<BM, BN, STAGES>(sched, args.ws, args.tickets, args.err, args.timeout, args.stall, args.early, args.trace);
 }
@@ -1615,6 +1622,21 @@ static int64_t tail_tiles(int64_t tiles, int64_t p) {
   return tiles >= p && 2 * r <= p ? r : 0;
 }
 
+// The accumulators that a launch's units sum their K blocks in, one after another (S = 1, 1-CTA tiles of up to 192
+// accumulator columns, fewer tiles than SMs: where split-K is the alternative).  An accumulator's error grows with its
+// K, about 1e-9 of the result per element, so a split's sums are the closer ones; with no more than 1024 of K to an
+// accumulator, one unsplit unit is as close, and the epilogue adds a finished accumulator while the MMAs fill the
+// next.  Error (2-norm, relative) on 128x64: 512 x 1736 x 2864 2.7e-6 -> 7.9e-7, 2176 x 384 x 2806 2.7e-6 -> 7.7e-7.
+static int32_t accum_segs(const rg_ctx* ctx, int32_t variant, int64_t rows, int64_t cols, int64_t depth) {
+  const TileKernel& tk = tile_kernel(variant_tile(variant));
+  if (variant_split(variant) > 1 || variant_streamk(variant) || variant_2sm(variant) ||
+      !segment_tile(tk.bm / 128 * tk.bn) ||
+      (rows + tk.bm - 1) / tk.bm * ((cols + tk.bn - 1) / tk.bn) >= ctx->sm_count)
+    return 1;
+  const int64_t kblocks = (depth + kBK - 1) / kBK;
+  return static_cast<int32_t>(std::min<int64_t>((kblocks + 15) / 16, 64));
+}
+
 struct Launch {
   KernFn fn = nullptr;
   CUtensorMap a, b, c, w;
@@ -1727,6 +1749,7 @@ static int prepare(rg_ctx* ctx, int64_t M, int64_t N, int64_t K, const void* A, 
   g.splits = sk ? static_cast<int32_t>(skg.tail_ctas) : splits;  // stream-K: CTAs sharing the tail tiles
   g.dp_tiles = sk ? static_cast<int32_t>(skg.dp_tiles) : 0;
   g.kblocks = static_cast<int32_t>(kblocks);
+  g.segs = accum_segs(ctx, variant, pm, pn, pk);
   g.whole = static_cast<int32_t>(tiles_m * tiles_n);
   if (splits == 1 && !sk && tk.bn % (two ? 256 : 128) == 0)
     g.whole -= static_cast<int32_t>(tail_tiles(tiles_m * tiles_n, two ? ctx->sm_count / 2 : ctx->sm_count));
@@ -1810,7 +1833,8 @@ static int plan_launches(rg_ctx* ctx, const rg_plan* plan, int64_t M, int64_t N,
     if (lf.m0 >= M || lf.n0 >= N || lf.k0 >= K) continue;  // wholly in the padding
     int64_t m0 = lf.m0, m = std::min(lf.m, M - m0), pm = lf.pm;
     const int64_t n = std::min(lf.n, N - lf.n0), k = std::min(lf.k, K - lf.k0);
-    if (m0 < row0 || m0 + m > row1) {
+    const bool part = m0 < row0 || m0 + m > row1;
+    if (part) {
       const int64_t end = std::min(m0 + m, row1);
       m0 = std::max(m0, row0);
       m = end - m0;
@@ -1823,6 +1847,10 @@ static int plan_launches(rg_ctx* ctx, const rg_plan* plan, int64_t M, int64_t N,
     Launch L;
     const int rc = prepare(ctx, m, n, k, a, lda, b, ldb, c, ldc, lf.variant, lf.beta, pm, lf.pn, lf.pk, &L);
     if (rc != RG_OK) return rc;
+    if (part) {  // rows of a leaf: summed as the whole leaf's
+      const int64_t rows = std::min(lf.m, M - lf.m0);
+      L.args.segs = accum_segs(ctx, lf.variant, lf.pm ? lf.pm : rows, lf.pn ? lf.pn : n, lf.pk ? lf.pk : k);
+    }
     out.push_back(L);
   }
   return RG_OK;
@@ -2799,7 +2827,7 @@ extern "C" int rg_gemm_grouped(rg_group* g, const rg_group_problem* probs, int32
     it.kblocks = a.kblocks;
     it.unit_start = static_cast<int32_t>(list.units[f]);
     it.splits = splits;
-    it.segs = serial ? a.splits : 1;
+    it.segs = serial ? a.splits : a.segs;
     it.ws_row0 = static_cast<int32_t>(my_rows > 0 ? row0 : 0);
     it.tk0 = static_cast<int32_t>(list.tickets);
     list.items[f].push_back(it);
