@@ -105,7 +105,7 @@ struct GemmArgs {
   int32_t dp_tiles;         // stream-K: tiles run whole before the shared tail
   int32_t panel;            // tile order: column panels of this many tiles (pairs: tile columns)
   int32_t early;            // 1: A and B are static, so loads may start before the preceding grid completes
-  int32_t segs;             // accumulators a unit's K blocks are summed in, one after another (see accum_segs)
+  int32_t subs;             // accumulators a unit's K blocks are summed in, one after another (see accum_subs)
   int32_t whole;            // (pair) tiles run whole, the rest as two half-width units each (see tail_tiles)
   float* ws;                // split-K partials [split][tile][BM][BN]
   int32_t* tickets;         // [tile][4], zero between launches
@@ -220,6 +220,8 @@ __device__ __forceinline__ void store_block(const CUtensorMap* tmC, const float 
 __host__ __device__ constexpr bool serial_tile(int acc_cols) { return acc_cols <= 128; }
 // Whether its units may sum their K blocks in several accumulators in turn (1-CTA tiles).
 __host__ __device__ constexpr bool segment_tile(int acc_cols) { return acc_cols <= 192; }
+// Whether its split-K units may as well (a thread then holds a split's sums beside those of all splits).
+__host__ __device__ constexpr bool segment_split_tile(int acc_cols) { return acc_cols <= 64; }
 
 // One work unit: which output tile of which problem, which K blocks, and where
 // its operands and output live.
@@ -238,8 +240,18 @@ struct Unit {
   int tk0 = 0;       // first ticket of the problem (grouped launches)
   bool half = false; // the unit is half of its tile's columns (tail tiles),
   int noff = 0;      // the left (0) or the right (1) one
-  int segs = 1;      // > 1: this unit runs all K splits of its tile, one accumulator after another (grouped launches)
+  // Accumulators the unit's K blocks are summed in, one after another: `segs` equal parts (grouped launches: all K
+  // splits of the tile; else 1) of `subs` equal parts each.
+  int segs = 1, subs = 1;
 };
+
+// K blocks of accumulator t of a unit that runs [kb0, kb1) in segs x subs of them
+__device__ __forceinline__ void sub_range(int kb0, int kb1, int segs, int subs, int t, int& lo, int& hi) {
+  const int g = t / subs, j = t - g * subs, n = kb1 - kb0;
+  const int a = kb0 + g * n / segs, b = kb0 + (g + 1) * n / segs;
+  lo = a + j * (b - a) / subs;
+  hi = a + (j + 1) * (b - a) / subs;
+}
 
 // Tile order: the tile grid is cut into column panels `panel` tiles wide and
 // walked row by row inside each panel, so the tiles resident at one time share a
@@ -299,7 +311,7 @@ struct SingleSched {
   const CUtensorMap* w;
   int tiles_m, tiles_n, splits, kblocks, M, N, beta;
   int whole = 0;
-  int segs = 1;
+  int subs = 1;
   int panel = 1 << 30;
   __device__ __forceinline__ void prefetch() const {
     prefetch_tmap(a);
@@ -322,7 +334,7 @@ struct SingleSched {
       x.half = u >= whole;
       x.noff = h & 1;
     }
-    if constexpr (!SPLIT) x.segs = segs;
+    x.subs = subs;
     return x;
   }
 };
@@ -353,6 +365,12 @@ template <class S, class = void>
 struct IsClusterSplit : std::false_type {};
 template <class S>
 struct IsClusterSplit<S, std::void_t<decltype(S::kClusterSplit)>> : std::bool_constant<S::kClusterSplit> {};
+
+// SingleSched itself, or a scheduler made from it
+template <class S>
+struct IsSingle
+    : std::bool_constant<std::is_base_of_v<SingleSched<false, false>, S> || std::is_base_of_v<SingleSched<false, true>, S> ||
+                         std::is_base_of_v<SingleSched<true, false>, S>> {};
 
 template <class S, class = void>
 struct HasTail : std::false_type {};
@@ -558,7 +576,7 @@ struct alignas(128) GroupItem {
   int32_t tiles_n, kblocks, unit_start, splits;
   int32_t ws_row0, tk0;
   int32_t segs;  // K splits one unit runs in turn (splits is then 1), or 1
-  int32_t reserved;
+  int32_t subs;  // accumulators of a split
 };
 struct alignas(128) GroupHeader {
   int32_t n_items;
@@ -589,7 +607,7 @@ struct GroupSched {
   int rank = 0, cid = 0, ncl = 1;
   // the calling warp's current item and its sizes (unit() is called by whole warps, in ascending order)
   mutable int cur = 0, loaded = -1;
-  mutable int4 d0, d1, d2;  // {M, N, beta, tiles_m}, {tiles_n, kblocks, unit_start, splits}, {ws_row0, tk0, segs, -}
+  mutable int4 d0, d1, d2;  // {M, N, beta, tiles_m}, {tiles_n, kblocks, unit_start, splits}, {ws_row0, tk0, segs, subs}
   __device__ __forceinline__ void prefetch() const {}
   __device__ __forceinline__ void init() {
     n_items = h->n_items;
@@ -670,6 +688,7 @@ struct GroupSched {
     x.ws_row0 = d2.x;
     x.tk0 = d2.y;
     x.segs = d2.z;
+    x.subs = d2.w;
     return x;
   }
 };
@@ -691,9 +710,12 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
   constexpr bool P2 = Sched::k2Sm;  // one CTA of a cta_group::2 pair
   constexpr bool CS = IsClusterSplit<Sched>::value;  // one K slice of a cluster split-K tile
   using C = KCfg<BM, BN, STAGES, P2 ? 2 : 1>;
-  // units may run all K splits of their tile (a thread then holds its sums of the whole tile in registers)
+  // units may sum several accumulators in turn (a thread then holds its sums of the whole tile in registers)
   constexpr bool SERIAL = Sched::kMapsInGlobal ? (P2 ? serial_tile(C::ACC_COLS) : segment_tile(C::ACC_COLS))
-                                               : !Sched::kSplit && !CS && !P2 && !Sched::kMemOnly && segment_tile(C::ACC_COLS);
+                          : IsSingle<Sched>::value && !CS && !Sched::kMemOnly
+                              ? (Sched::kSplit ? segment_split_tile(C::ACC_COLS) : segment_tile(C::ACC_COLS))
+                              : false;
+  constexpr bool SUBS_SPLIT = SERIAL && Sched::kSplit && !P2 && segment_split_tile(C::ACC_COLS);
   constexpr bool TAIL = HasTail<Sched>::value;  // units may be halves of their tile's columns
   static_assert(!TAIL || C::HALVABLE, "tail tiles");
   extern __shared__ uint8_t smem_raw[];
@@ -849,20 +871,21 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
     // a pair's odd CTA issues nothing: the even CTA's MMAs read and write both
     const int issue_units = (!P2 || sched.rank == 0) ? nunits : 0;
     // the K range and segments of the next unit, looked up while the current one's MMAs run
-    int kb0n = 0, kb1n = 0, segsn = 1;
+    int kb0n = 0, kb1n = 0, segsn = 1, subsn = 1;
     uint32_t idesc = C::IDESC;
     if (issue_units > 0) {
       const Unit w = sched.unit(0);
       kb0n = w.kb0;
       kb1n = w.kb1;
       segsn = w.segs;
+      subsn = w.subs;
       if (TAIL && w.half) idesc = C::IDESC_HALF;
     }
     int seg = 0;
     for (int i = 0; ok && i < issue_units;) {
-      // the unit's K blocks, or those of its K split `seg`
-      const int kb0 = SERIAL && segsn > 1 ? seg * kb1n / segsn : kb0n;
-      const int kb1 = SERIAL && segsn > 1 ? (seg + 1) * kb1n / segsn : kb1n;
+      // the unit's K blocks, or those of its accumulator `seg`
+      int kb0 = kb0n, kb1 = kb1n;
+      if (SERIAL && segsn * subsn > 1) sub_range(kb0n, kb1n, segsn, subsn, seg, kb0, kb1);
       ok = mbar_wait_warp(tempty_bar(acc), aph ^ 1u, timeout, abort_flag);
       if (!ok) break;
       tc_fence_after();
@@ -904,13 +927,14 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
         acc = 0;
         aph ^= 1u;
       }
-      if (SERIAL && ++seg < segsn) continue;
+      if (SERIAL && ++seg < segsn * subsn) continue;
       seg = 0;
       if (++i < issue_units) {
         const Unit w = sched.unit(i);
         kb0n = w.kb0;
         kb1n = w.kb1;
         segsn = w.segs;
+        subsn = w.subs;
         if (TAIL && w.half) idesc = C::IDESC_HALF;
       } else if (lane == 0) {
         RG_STAMP(5);
@@ -940,6 +964,65 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
     int acc = 0, sbuf = 0;
     uint32_t aph = 0;
     bool ok = true;
+    // The sum of the unit's accumulators, the first of which is ready; the last is left to be released.
+    auto sum_accumulators = [&](const Unit& w, int& acc, uint32_t& aph, float (&sum)[C::ACC_COLS / 32][32]) {
+      // a split's sums beside those of the splits before it: one and the same where a split is one accumulator
+      constexpr bool TWO_LEVEL = SUBS_SPLIT && Sched::kMapsInGlobal;
+      float part[TWO_LEVEL ? C::ACC_COLS / 32 : 1][32];
+      // -0 is the sum's neutral element (-0 + x = x, also for x = -0)
+#pragma unroll
+      for (int c = 0; c < C::ACC_COLS / 32; ++c)
+#pragma unroll
+        for (int e = 0; e < 32; ++e) {
+          sum[c][e] = -0.f;
+          if constexpr (TWO_LEVEL) part[c][e] = -0.f;
+        }
+      const int n = w.segs * w.subs;
+#pragma unroll 1
+      for (int seg = 0; seg < n; ++seg) {
+        if (seg > 0) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) {
+            if constexpr (P2)
+              mbar_arrive_cluster(mapa_shared(tempty_bar(acc), 0));
+            else
+              mbar_arrive(tempty_bar(acc));
+          }
+          if (++acc == C::NBUF) {
+            acc = 0;
+            aph ^= 1u;
+          }
+          if (!mbar_wait_warp(tfull_bar(acc), aph, timeout, abort_flag)) return false;
+          tc_fence_after();
+        }
+        int lo, hi;
+        sub_range(w.kb0, w.kb1, w.segs, w.subs, seg, lo, hi);
+        const bool some = hi > lo;  // the accumulator has K blocks
+        const uint32_t t = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * C::ACC_COLS);
+        const bool end = !TWO_LEVEL || (seg + 1) % w.subs == 0;  // the last accumulator of its split
+#pragma unroll
+        for (int c = 0; c < C::ACC_COLS / 32; ++c) {
+          uint32_t v[32];
+          tmem_ld_32x32b_x32(t + c * 32, v);
+          tmem_ld_wait_for(v);
+#pragma unroll
+          for (int e = 0; e < 32; ++e) {
+            const float x = some ? __uint_as_float(v[e]) : 0.f;
+            if constexpr (TWO_LEVEL) {
+              part[c][e] += x;
+              if (end) {
+                sum[c][e] += part[c][e];
+                part[c][e] = -0.f;
+              }
+            } else {
+              sum[c][e] += x;
+            }
+          }
+        }
+      }
+      return true;
+    };
     for (int i = 0; i < nunits; ++i) {
       const Unit w = sched.unit(i);
       const int tile = w.tile, s = w.s, tm = w.tm, tn = w.tn, kb0 = w.kb0, kb1 = w.kb1, ntiles = w.ntiles;
@@ -1018,49 +1101,15 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
           store_block(w.c, sum, tm * BM + (j / kCols) * 128 + q * 32, tn * BN + (j % kCols) * 32, w.M, w.N, w.beta,
                       stg0, sbuf, lane);
         }
-      } else if (SERIAL && w.segs > 1) {
-        // All K splits of the tile, one accumulator after another: their sum in the order
-        // 0..S-1, as the workspace path's last arriver forms it, without the partials' round
-        // trip through memory (publishing, waiting for and re-reading a split's partial takes an
+      } else if (SERIAL && (w.segs > 1 || (w.subs > 1 && (!SUBS_SPLIT || w.splits == 1)))) {
+        // Several accumulators, one after another, summed in registers: all K splits of the tile (their sum in the
+        // order 0..S-1, as the workspace path's last arriver forms it, without the partials' round
+        // trip through memory; publishing, waiting for and re-reading a split's partial takes an
         // epilogue warp 3-6 us: 8 problems of 512 x 576 x 1024 on 128x64, S = 4, 59.5 us; without
-        // a split 18.5).
+        // a split 18.5), each in `subs` accumulators.
         if constexpr (SERIAL) {
-          // -0 is the sum's neutral element (-0 + x = x, also for x = -0)
           float sum[C::ACC_COLS / 32][32];
-#pragma unroll
-          for (int c = 0; c < C::ACC_COLS / 32; ++c)
-#pragma unroll
-            for (int e = 0; e < 32; ++e) sum[c][e] = -0.f;
-#pragma unroll 1
-          for (int seg = 0; seg < w.segs; ++seg) {
-            if (seg > 0) {
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) {
-                if constexpr (P2)
-                  mbar_arrive_cluster(mapa_shared(tempty_bar(acc), 0));
-                else
-                  mbar_arrive(tempty_bar(acc));
-              }
-              if (++acc == C::NBUF) {
-                acc = 0;
-                aph ^= 1u;
-              }
-              ok = mbar_wait_warp(tfull_bar(acc), aph, timeout, abort_flag);
-              if (!ok) break;
-              tc_fence_after();
-            }
-            const bool some = (seg + 1) * kb1 / w.segs > seg * kb1 / w.segs;  // the split has K blocks
-            const uint32_t t = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * C::ACC_COLS);
-#pragma unroll
-            for (int c = 0; c < C::ACC_COLS / 32; ++c) {
-              uint32_t v[32];
-              tmem_ld_32x32b_x32(t + c * 32, v);
-              tmem_ld_wait_for(v);
-#pragma unroll
-              for (int e = 0; e < 32; ++e) sum[c][e] += some ? __uint_as_float(v[e]) : 0.f;
-            }
-          }
+          ok = sum_accumulators(w, acc, aph, sum);
           if (!ok) break;
 #pragma unroll
           for (int c = 0; c < C::ACC_COLS / 32; ++c)
@@ -1083,14 +1132,27 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
         // for the stores, fence them against the generic proxy and take the ticket
         // of this (tile, warp) row block with an acquire-release atomic.
         const int wrow = w.ws_row0 + (s * ntiles + tile) * BM;
-#pragma unroll 1
-        for (int h = 0; h < C::HALVES; ++h)
-#pragma unroll 1
-          for (int c = 0; c < BN / 32; ++c) {
-            float v[32];
-            load_acc(tacc + h * BN + c * 32, have, v);
-            store_block(w.w, v, wrow + h * 128 + q * 32, c * 32, INT_MAX, INT_MAX, 0, stg0, sbuf, lane);
+        const bool subs = SUBS_SPLIT && w.subs > 1;  // the split's sum is then in registers, not in TMEM
+        if (subs) {
+          if constexpr (SUBS_SPLIT) {
+            float sum[C::ACC_COLS / 32][32];
+            ok = sum_accumulators(w, acc, aph, sum);
+            if (!ok) break;
+#pragma unroll
+            for (int c = 0; c < C::ACC_COLS / 32; ++c)
+              store_block(w.w, sum[c], wrow + (c * 32 / BN) * 128 + q * 32, c * 32 % BN, INT_MAX, INT_MAX, 0, stg0, sbuf,
+                          lane);
           }
+        } else {
+#pragma unroll 1
+          for (int h = 0; h < C::HALVES; ++h)
+#pragma unroll 1
+            for (int c = 0; c < BN / 32; ++c) {
+              float v[32];
+              load_acc(tacc + h * BN + c * 32, have, v);
+              store_block(w.w, v, wrow + h * 128 + q * 32, c * 32, INT_MAX, INT_MAX, 0, stg0, sbuf, lane);
+            }
+        }
         if (lane == 0) {
           bulk_wait<0>();
           fence_proxy_async_global();
@@ -1118,7 +1180,7 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
           // one row per lane) is brought into that layout through the staging buffer.
           constexpr int kBatch = 3;
           const int rsub = lane >> 3, g = lane & 7;
-          if (w.splits == 2) {
+          if (w.splits == 2 && !subs) {
             // Two pieces (split 2, every stream-K tail tile): the other piece's partial of the
             // next 32 x 32 block is loaded while this block is reduced, hiding the load latency;
             // own + other is the same sum in either order, so the result is that of the fixed order.
@@ -1211,7 +1273,7 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
 #pragma unroll
                 for (int b = 0; b < kBatch; ++b) {
                   const int tb = base + b;
-                  if (tb < w.splits && tb != s) {
+                  if (tb < w.splits && (tb != s || subs)) {  // (its own as well, where TMEM does not hold it)
                     const float* src = ws + static_cast<size_t>(w.ws_row0 + (tb * ntiles + tile) * BM + h * 128 +
                                                                 q * 32) * BN + c * 32 + 4 * g;
 #pragma unroll
@@ -1225,7 +1287,7 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
                   if (tb < w.splits) {
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
-                      const float4 p = (tb == s) ? o[j] : x[b][j];
+                      const float4 p = (tb == s && !subs) ? o[j] : x[b][j];
                       if (t == 0) {
                         sum[j] = p;
                       } else {
@@ -1314,7 +1376,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   SingleSched<SPLIT, !SPLIT && KCfg<BM, BN, STAGES>::HALVABLE> sched{
       &tmA, &tmB, &tmC, &tmW, args.tiles_m, args.tiles_n, args.splits, args.kblocks, args.M, args.N, args.beta};
   sched.whole = args.whole;
-  sched.segs = args.segs;
+  sched.subs = args.subs;
   sched.panel = args.panel;
   gemm_body<BM, BN, STAGES>(sched, args.ws, args.tickets, args.err, args.timeout, args.stall, args.early, args.trace);
 }
@@ -1622,18 +1684,20 @@ static int64_t tail_tiles(int64_t tiles, int64_t p) {
   return tiles >= p && 2 * r <= p ? r : 0;
 }
 
-// The accumulators that a launch's units sum their K blocks in, one after another (S = 1, 1-CTA tiles of up to 192
-// accumulator columns, fewer tiles than SMs: where split-K is the alternative).  An accumulator's error grows with its
-// K, about 1e-9 of the result per element, so a split's sums are the closer ones; with no more than 1024 of K to an
-// accumulator, one unsplit unit is as close, and the epilogue adds a finished accumulator while the MMAs fill the
-// next.  Error (2-norm, relative) on 128x64: 512 x 1736 x 2864 2.7e-6 -> 7.9e-7, 2176 x 384 x 2806 2.7e-6 -> 7.7e-7.
-static int32_t accum_segs(const rg_ctx* ctx, int32_t variant, int64_t rows, int64_t cols, int64_t depth) {
+// The accumulators that a launch's units sum their K blocks in, one after another (1-CTA tiles of up to 192
+// accumulator columns; of 64 with split-K; fewer tiles than SMs, where split-K is an alternative).  An accumulator's
+// error grows with its K, about 1e-9 of the result per element, so the variant with the most splits has the closest
+// sums; with no more than 1024 of K to an accumulator the others are as close, and the epilogue adds a finished
+// accumulator while the MMAs fill the next.  Error (2-norm, relative) on 128x64: 512 x 1736 x 2864 2.7e-6 -> 7.9e-7,
+// 2176 x 384 x 2806 2.7e-6 -> 7.7e-7, and with S = 2 16 x 1152 x 3953 1.8e-6 -> 8.3e-7.
+static int32_t accum_subs(const rg_ctx* ctx, int32_t variant, int64_t rows, int64_t cols, int64_t depth) {
   const TileKernel& tk = tile_kernel(variant_tile(variant));
-  if (variant_split(variant) > 1 || variant_streamk(variant) || variant_2sm(variant) ||
-      !segment_tile(tk.bm / 128 * tk.bn) ||
+  const int splits = variant_split(variant), acc_cols = tk.bm / 128 * tk.bn;
+  if (variant_streamk(variant) || variant_2sm(variant) ||
+      !(splits > 1 ? segment_split_tile(acc_cols) : segment_tile(acc_cols)) ||
       (rows + tk.bm - 1) / tk.bm * ((cols + tk.bn - 1) / tk.bn) >= ctx->sm_count)
     return 1;
-  const int64_t kblocks = (depth + kBK - 1) / kBK;
+  const int64_t kblocks = ((depth + kBK - 1) / kBK + splits - 1) / splits;
   return static_cast<int32_t>(std::min<int64_t>((kblocks + 15) / 16, 64));
 }
 
@@ -1749,7 +1813,7 @@ static int prepare(rg_ctx* ctx, int64_t M, int64_t N, int64_t K, const void* A, 
   g.splits = sk ? static_cast<int32_t>(skg.tail_ctas) : splits;  // stream-K: CTAs sharing the tail tiles
   g.dp_tiles = sk ? static_cast<int32_t>(skg.dp_tiles) : 0;
   g.kblocks = static_cast<int32_t>(kblocks);
-  g.segs = accum_segs(ctx, variant, pm, pn, pk);
+  g.subs = accum_subs(ctx, variant, pm, pn, pk);
   g.whole = static_cast<int32_t>(tiles_m * tiles_n);
   if (splits == 1 && !sk && tk.bn % (two ? 256 : 128) == 0)
     g.whole -= static_cast<int32_t>(tail_tiles(tiles_m * tiles_n, two ? ctx->sm_count / 2 : ctx->sm_count));
@@ -1849,7 +1913,7 @@ static int plan_launches(rg_ctx* ctx, const rg_plan* plan, int64_t M, int64_t N,
     if (rc != RG_OK) return rc;
     if (part) {  // rows of a leaf: summed as the whole leaf's
       const int64_t rows = std::min(lf.m, M - lf.m0);
-      L.args.segs = accum_segs(ctx, lf.variant, lf.pm ? lf.pm : rows, lf.pn ? lf.pn : n, lf.pk ? lf.pk : k);
+      L.args.subs = accum_subs(ctx, lf.variant, lf.pm ? lf.pm : rows, lf.pn ? lf.pn : n, lf.pk ? lf.pk : k);
     }
     out.push_back(L);
   }
@@ -2827,7 +2891,8 @@ extern "C" int rg_gemm_grouped(rg_group* g, const rg_group_problem* probs, int32
     it.kblocks = a.kblocks;
     it.unit_start = static_cast<int32_t>(list.units[f]);
     it.splits = splits;
-    it.segs = serial ? a.splits : a.segs;
+    it.segs = serial ? a.splits : 1;
+    it.subs = a.subs;
     it.ws_row0 = static_cast<int32_t>(my_rows > 0 ? row0 : 0);
     it.tk0 = static_cast<int32_t>(list.tickets);
     list.items[f].push_back(it);
