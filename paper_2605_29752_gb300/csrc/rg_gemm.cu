@@ -219,8 +219,8 @@ __device__ __forceinline__ void store_block(const CUtensorMap* tmC, const float 
 // then hold one FP32 sum per accumulator column (TMEM columns: BN, twice that for 256-row CTAs).
 __host__ __device__ constexpr bool serial_tile(int acc_cols) { return acc_cols <= 128; }
 // Whether its units may sum their K blocks in several accumulators in turn (1-CTA tiles).
-__host__ __device__ constexpr bool segment_tile(int acc_cols) { return acc_cols <= 192; }
-// Whether its split-K units may as well (a thread then holds a split's sums beside those of all splits).
+__host__ __device__ constexpr bool segment_tile(int acc_cols) { return acc_cols <= 128; }
+// Whether its split-K units may as well.
 __host__ __device__ constexpr bool segment_split_tile(int acc_cols) { return acc_cols <= 64; }
 
 // One work unit: which output tile of which problem, which K blocks, and where
@@ -240,17 +240,15 @@ struct Unit {
   int tk0 = 0;       // first ticket of the problem (grouped launches)
   bool half = false; // the unit is half of its tile's columns (tail tiles),
   int noff = 0;      // the left (0) or the right (1) one
-  // Accumulators the unit's K blocks are summed in, one after another: `segs` equal parts (grouped launches: all K
-  // splits of the tile; else 1) of `subs` equal parts each.
+  // Accumulators the unit's K blocks are summed in, one after another: all K splits of the tile (grouped launches), or
+  // `subs` equal parts; one of the two is 1.
   int segs = 1, subs = 1;
 };
 
-// K blocks of accumulator t of a unit that runs [kb0, kb1) in segs x subs of them
-__device__ __forceinline__ void sub_range(int kb0, int kb1, int segs, int subs, int t, int& lo, int& hi) {
-  const int g = t / subs, j = t - g * subs, n = kb1 - kb0;
-  const int a = kb0 + g * n / segs, b = kb0 + (g + 1) * n / segs;
-  lo = a + j * (b - a) / subs;
-  hi = a + (j + 1) * (b - a) / subs;
+// K blocks of accumulator t of n of a unit that runs [kb0, kb1)  (32-bit: t < 64 and kb1 <= 2^24)
+__device__ __forceinline__ void sub_range(int kb0, int kb1, int n, int t, int& lo, int& hi) {
+  lo = kb0 + t * (kb1 - kb0) / n;
+  hi = kb0 + (t + 1) * (kb1 - kb0) / n;
 }
 
 // Tile order: the tile grid is cut into column panels `panel` tiles wide and
@@ -885,7 +883,7 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
     for (int i = 0; ok && i < issue_units;) {
       // the unit's K blocks, or those of its accumulator `seg`
       int kb0 = kb0n, kb1 = kb1n;
-      if (SERIAL && segsn * subsn > 1) sub_range(kb0n, kb1n, segsn, subsn, seg, kb0, kb1);
+      if (SERIAL && segsn * subsn > 1) sub_range(kb0n, kb1n, segsn * subsn, seg, kb0, kb1);
       ok = mbar_wait_warp(tempty_bar(acc), aph ^ 1u, timeout, abort_flag);
       if (!ok) break;
       tc_fence_after();
@@ -966,17 +964,11 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
     bool ok = true;
     // The sum of the unit's accumulators, the first of which is ready; the last is left to be released.
     auto sum_accumulators = [&](const Unit& w, int& acc, uint32_t& aph, float (&sum)[C::ACC_COLS / 32][32]) {
-      // a split's sums beside those of the splits before it: one and the same where a split is one accumulator
-      constexpr bool TWO_LEVEL = SUBS_SPLIT && Sched::kMapsInGlobal;
-      float part[TWO_LEVEL ? C::ACC_COLS / 32 : 1][32];
       // -0 is the sum's neutral element (-0 + x = x, also for x = -0)
 #pragma unroll
       for (int c = 0; c < C::ACC_COLS / 32; ++c)
 #pragma unroll
-        for (int e = 0; e < 32; ++e) {
-          sum[c][e] = -0.f;
-          if constexpr (TWO_LEVEL) part[c][e] = -0.f;
-        }
+        for (int e = 0; e < 32; ++e) sum[c][e] = -0.f;
       const int n = w.segs * w.subs;
 #pragma unroll 1
       for (int seg = 0; seg < n; ++seg) {
@@ -997,28 +989,16 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
           tc_fence_after();
         }
         int lo, hi;
-        sub_range(w.kb0, w.kb1, w.segs, w.subs, seg, lo, hi);
+        sub_range(w.kb0, w.kb1, n, seg, lo, hi);
         const bool some = hi > lo;  // the accumulator has K blocks
         const uint32_t t = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * C::ACC_COLS);
-        const bool end = !TWO_LEVEL || (seg + 1) % w.subs == 0;  // the last accumulator of its split
 #pragma unroll
         for (int c = 0; c < C::ACC_COLS / 32; ++c) {
           uint32_t v[32];
           tmem_ld_32x32b_x32(t + c * 32, v);
           tmem_ld_wait_for(v);
 #pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            const float x = some ? __uint_as_float(v[e]) : 0.f;
-            if constexpr (TWO_LEVEL) {
-              part[c][e] += x;
-              if (end) {
-                sum[c][e] += part[c][e];
-                part[c][e] = -0.f;
-              }
-            } else {
-              sum[c][e] += x;
-            }
-          }
+          for (int e = 0; e < 32; ++e) sum[c][e] += some ? __uint_as_float(v[e]) : 0.f;
         }
       }
       return true;
@@ -1031,7 +1011,7 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
       if (i == 0 && warp == 2 && lane == 0) RG_STAMP(6);
       tc_fence_after();
       const bool have = kb1 > kb0;
-      const uint32_t tacc = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * C::ACC_COLS);
+      uint32_t tacc = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * C::ACC_COLS);
       if constexpr (CS) {
         // Split-K inside the cluster, through distributed shared memory.  Block b = q kPerWarp + j
         // (32 x 32, j = h kCols + c) of the tile is reduced by CTA b % S; the other CTAs write their
@@ -1106,7 +1086,7 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
         // order 0..S-1, as the workspace path's last arriver forms it, without the partials' round
         // trip through memory; publishing, waiting for and re-reading a split's partial takes an
         // epilogue warp 3-6 us: 8 problems of 512 x 576 x 1024 on 128x64, S = 4, 59.5 us; without
-        // a split 18.5), each in `subs` accumulators.
+        // a split 18.5), or the unit's `subs` parts.
         if constexpr (SERIAL) {
           float sum[C::ACC_COLS / 32][32];
           ok = sum_accumulators(w, acc, aph, sum);
@@ -1132,27 +1112,25 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
         // for the stores, fence them against the generic proxy and take the ticket
         // of this (tile, warp) row block with an acquire-release atomic.
         const int wrow = w.ws_row0 + (s * ntiles + tile) * BM;
-        const bool subs = SUBS_SPLIT && w.subs > 1;  // the split's sum is then in registers, not in TMEM
-        if (subs) {
-          if constexpr (SUBS_SPLIT) {
+        if constexpr (SUBS_SPLIT) {
+          if (w.subs > 1) {  // the split's sum takes the place of its last accumulator
             float sum[C::ACC_COLS / 32][32];
             ok = sum_accumulators(w, acc, aph, sum);
             if (!ok) break;
+            tacc = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * C::ACC_COLS);
 #pragma unroll
-            for (int c = 0; c < C::ACC_COLS / 32; ++c)
-              store_block(w.w, sum[c], wrow + (c * 32 / BN) * 128 + q * 32, c * 32 % BN, INT_MAX, INT_MAX, 0, stg0, sbuf,
-                          lane);
+            for (int c = 0; c < C::ACC_COLS / 32; ++c) tmem_st_32x32b_x32(tacc + c * 32, sum[c]);
+            tmem_st_wait();
           }
-        } else {
-#pragma unroll 1
-          for (int h = 0; h < C::HALVES; ++h)
-#pragma unroll 1
-            for (int c = 0; c < BN / 32; ++c) {
-              float v[32];
-              load_acc(tacc + h * BN + c * 32, have, v);
-              store_block(w.w, v, wrow + h * 128 + q * 32, c * 32, INT_MAX, INT_MAX, 0, stg0, sbuf, lane);
-            }
         }
+#pragma unroll 1
+        for (int h = 0; h < C::HALVES; ++h)
+#pragma unroll 1
+          for (int c = 0; c < BN / 32; ++c) {
+            float v[32];
+            load_acc(tacc + h * BN + c * 32, have, v);
+            store_block(w.w, v, wrow + h * 128 + q * 32, c * 32, INT_MAX, INT_MAX, 0, stg0, sbuf, lane);
+          }
         if (lane == 0) {
           bulk_wait<0>();
           fence_proxy_async_global();
@@ -1180,7 +1158,7 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
           // one row per lane) is brought into that layout through the staging buffer.
           constexpr int kBatch = 3;
           const int rsub = lane >> 3, g = lane & 7;
-          if (w.splits == 2 && !subs) {
+          if (w.splits == 2) {
             // Two pieces (split 2, every stream-K tail tile): the other piece's partial of the
             // next 32 x 32 block is loaded while this block is reduced, hiding the load latency;
             // own + other is the same sum in either order, so the result is that of the fixed order.
@@ -1273,7 +1251,7 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
 #pragma unroll
                 for (int b = 0; b < kBatch; ++b) {
                   const int tb = base + b;
-                  if (tb < w.splits && (tb != s || subs)) {  // (its own as well, where TMEM does not hold it)
+                  if (tb < w.splits && tb != s) {
                     const float* src = ws + static_cast<size_t>(w.ws_row0 + (tb * ntiles + tile) * BM + h * 128 +
                                                                 q * 32) * BN + c * 32 + 4 * g;
 #pragma unroll
@@ -1287,7 +1265,7 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
                   if (tb < w.splits) {
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
-                      const float4 p = (tb == s && !subs) ? o[j] : x[b][j];
+                      const float4 p = (tb == s) ? o[j] : x[b][j];
                       if (t == 0) {
                         sum[j] = p;
                       } else {
@@ -1684,7 +1662,7 @@ static int64_t tail_tiles(int64_t tiles, int64_t p) {
   return tiles >= p && 2 * r <= p ? r : 0;
 }
 
-// The accumulators that a launch's units sum their K blocks in, one after another (1-CTA tiles of up to 192
+// The accumulators that a launch's units sum their K blocks in, one after another (1-CTA tiles of up to 128
 // accumulator columns; of 64 with split-K; fewer tiles than SMs, where split-K is an alternative).  An accumulator's
 // error grows with its K, about 1e-9 of the result per element, so the variant with the most splits has the closest
 // sums; with no more than 1024 of K to an accumulator the others are as close, and the epilogue adds a finished
@@ -2847,7 +2825,7 @@ extern "C" int rg_gemm_grouped(rg_group* g, const rg_group_problem* probs, int32
   // The K splits of a tile as one unit, where that is no longer than a CTA's (cluster's) share of
   // the family's K blocks: splitting then only adds the partials' traffic, not parallelism.
   auto serial_splits = [&](const Prepared& q) {
-    return q.L.args.splits > 1 && rg::serial_tile(rg::family_bn(q.family) * (cta_rows(q.family) / 128)) &&
+    return q.L.args.splits > 1 && q.L.args.subs == 1 && rg::serial_tile(rg::family_bn(q.family) * (cta_rows(q.family) / 128)) &&
            q.L.args.kblocks * sharers(q.family) <= blocks[q.family];
   };
   for (const auto& q : prep) {  // partials and tickets of the other splits

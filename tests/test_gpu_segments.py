@@ -24,7 +24,7 @@ def ctx(rg):
 
 # K: one accumulator up to 1024; 2 of 8 or 9 and of 16 blocks, 4 with a ragged last block, 8
 @pytest.mark.parametrize("K, segs", [(1024, 1), (1032, 2), (2048, 2), (3100, 4), (8000, 8)])
-@pytest.mark.parametrize("tile", [0, 1, 3, 6])
+@pytest.mark.parametrize("tile", [0, 1, 3])
 @pytest.mark.parametrize("M, N, beta", [(1, 8, 0), (300, 392, 1), (1000, 1096, 0)])
 def test_segments(rg, ctx, tile, M, N, beta, K, segs):
     ldk = -(-K // 8) * 8
@@ -43,8 +43,8 @@ def test_segments(rg, ctx, tile, M, N, beta, K, segs):
         rg.rg_group_destroy(g)
 
 
-# 128x64 with split-K and K beyond 1024 to a split: alone, in a grouped call that splits as well (one problem) and in one
-# that fills the chip, whose units run all splits in turn; each split's sum is that of its accumulators, in order
+# 128x64 with split-K and K beyond 1024 to a split: alone, in a grouped call of one problem and in one
+# that fills the chip; each split's sum is that of its accumulators, in order
 @pytest.mark.parametrize("split, K", [(2, 2049), (2, 4096), (4, 5000), (8, 9000)])
 @pytest.mark.parametrize("M, N, beta", [(1, 8, 0), (300, 392, 1), (512, 1024, 0)])
 def test_split_segments(rg, ctx, split, K, M, N, beta):
@@ -73,7 +73,7 @@ def test_split_segments(rg, ctx, split, K, M, N, beta):
     assert subs > 1 and torch.equal(C, R)
     g = rg.rg_group_create(ctx, 1, 64, 64 << 20)
     try:
-        for n in (1, 40):  # 40 problems: K blocks enough for every CTA to run its tiles whole
+        for n in (1, 40):  # 40 problems: K blocks enough for every CTA
             outs = [c0.clone() for _ in range(n)]
             rg.rg_gemm_grouped(g, rg.group_problems([(M, N, K, A, ldk, B, N, G, N, beta, 0, 0, 0, v) for G in outs]), n)
             rg.rg_check(ctx)
