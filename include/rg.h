@@ -275,7 +275,9 @@ int rg_gemm_plan(rg_ctx* ctx, const rg_plan* plan, int64_t M, int64_t N, int64_t
  * copies A (M x K, lda) and B (K x N, ldb) from the host into device staging
  * buffers the context owns (allocated on first use and grown when a larger
  * problem comes; leading dimensions rounded up to the TMA alignment there),
- * executes the plan on `stream`, copies C (M x N, ldc) back and synchronises
+ * executes the plan on `stream`, copies C (M x N, ldc) back (large page-locked
+ * operands of one block each: in row panels, whose copies run on streams of the
+ * context beside the GEMMs, with the same result) and synchronises
  * the stream, so C holds the result on return.  Host buffers may be pageable
  * or pinned (pinned memory makes the copies asynchronous DMA).  M, N, K > 0.
  * Errors: those of rg_gemm_plan, RG_ERR_OOM for a staging buffer,
