@@ -1616,21 +1616,29 @@ struct rg_ctx {
 namespace rg {
 
 static PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
+static PFN_cuPointerGetAttribute_v4000 g_pointer_attribute = nullptr;
 static std::mutex g_mu;
 
 static int cuda_fail(cudaError_t e, const char* what) {
   return fail(RG_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
+// The driver functions the library calls itself.
 static int get_encode() {
   std::lock_guard<std::mutex> lk(g_mu);
-  if (g_encode) return RG_OK;
-  void* fn = nullptr;
-  cudaDriverEntryPointQueryResult q;
-  cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q);
-  if (e != cudaSuccess || q != cudaDriverEntryPointSuccess || !fn)
-    return fail(RG_ERR_CUDA, "cannot resolve cuTensorMapEncodeTiled from the driver");
-  g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
+  if (g_encode && g_pointer_attribute) return RG_OK;
+  auto resolve = [](const char* name, unsigned version) -> void* {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion(name, &fn, version, cudaEnableDefault, &q);
+    return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? fn : nullptr;
+  };
+  void* encode = resolve("cuTensorMapEncodeTiled", 12000);
+  void* attribute = resolve("cuPointerGetAttribute", 4000);
+  if (!encode || !attribute)
+    return fail(RG_ERR_CUDA, "cannot resolve cuTensorMapEncodeTiled and cuPointerGetAttribute from the driver");
+  g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(encode);
+  g_pointer_attribute = reinterpret_cast<PFN_cuPointerGetAttribute_v4000>(attribute);
   return RG_OK;
 }
 
@@ -2219,18 +2227,19 @@ int grow_stage(void** buf, int64_t* cap, int64_t bytes, cudaStream_t st) {
   return RG_OK;
 }
 
-// Whether the device can read [p, p + bytes) itself: page-locked host memory at its own address.
+// Whether the device can read [p, p + bytes) itself: page-locked host memory at its own address, all of it of one
+// allocation or registration (between two registrations there may be pages that the SMs cannot read).
 bool pinned(const void* p, int64_t bytes) {
-  const auto* c = static_cast<const unsigned char*>(p);
-  for (const unsigned char* at : {c, c + bytes - 1}) {
-    cudaPointerAttributes a{};
-    if (cudaPointerGetAttributes(&a, at) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    if (a.type != cudaMemoryTypeHost || a.devicePointer != at) return false;
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
   }
-  return true;
+  if (a.type != cudaMemoryTypeHost || a.devicePointer != p) return false;
+  return rg::in_one_block(reinterpret_cast<uintptr_t>(p), bytes, [](uintptr_t at, uintptr_t* start, size_t* size) {
+    return rg::g_pointer_attribute(start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, at) == CUDA_SUCCESS &&
+           rg::g_pointer_attribute(size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, at) == CUDA_SUCCESS;
+  });
 }
 
 // Rows of a host matrix to a staging buffer (16-byte aligned, its pitch a multiple of 16): by a copy engine where

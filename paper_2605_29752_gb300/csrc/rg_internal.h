@@ -1,6 +1,7 @@
 // Internal declarations shared by the library's translation units.
 #pragma once
 
+#include <cstddef>
 #include <cstdint>
 #include <string>
 #include <vector>
@@ -23,6 +24,18 @@ inline bool grid_valid(const rg_grid& g) {
   return true;
 }
 inline int64_t axis_value(const rg_axis& a, int64_t i) { return a.start + i * a.step; }
+
+// Whether [p, p + bytes) is one block of memory: `block(p, &start, &size)` gives the allocation or registration that
+// an address belongs to, or false where there is none.  Two ends in blocks of their own do not make what lies between
+// them one.
+template <class Block>
+bool in_one_block(uintptr_t p, int64_t bytes, Block block) {
+  uintptr_t start = 0;
+  size_t size = 0;
+  if (bytes <= 0 || !block(p, &start, &size) || p < start) return false;
+  const uint64_t before = p - start;
+  return before <= size && static_cast<uint64_t>(bytes) <= size - before;
+}
 
 struct Plan {
   rg_grid grid{};
