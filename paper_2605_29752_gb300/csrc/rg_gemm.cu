@@ -1444,9 +1444,11 @@ __global__ void __launch_bounds__(kCopyThreads) group_copy_kernel(const uint4* _
   for (i += step; i < n; i += step) dev[i] = host[i];
 }
 
+// `list` is written by the copy while these kernels are already running (they wait for it first), so it is no
+// __restrict__ pointer: its bytes are not constant over the kernel, and must not be read as if they were.
 template <int BM, int BN, int STAGES>
 __global__ void __launch_bounds__(kThreads, 1)
-    gemm_bf16_grouped_kernel(const unsigned char* __restrict__ list, int family,
+    gemm_bf16_grouped_kernel(const unsigned char* list, int family,
                              const __grid_constant__ CUtensorMap tmW, float* ws, int32_t* tickets, int32_t* err,
                              long long timeout) {
   grid_dependency_wait();  // the list has been copied
@@ -1460,7 +1462,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // two CTAs, so a graph kernel node launches it as pairs without a launch attribute.
 template <int BN, int STAGES>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-    gemm_bf16_grouped_2sm_kernel(const unsigned char* __restrict__ list, int family,
+    gemm_bf16_grouped_2sm_kernel(const unsigned char* list, int family,
                                  const __grid_constant__ CUtensorMap tmW, float* ws, int32_t* tickets, int32_t* err,
                                  long long timeout) {
   grid_dependency_wait();  // the list has been copied
