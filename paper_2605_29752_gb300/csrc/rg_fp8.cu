@@ -641,10 +641,12 @@ __device__ __forceinline__ uint32_t e4m3x4(float a, float b, float c, float d) {
 // rate); 8192^2: 309 -> 50.4, 98 % of that rate.  512 threads are the faster where the blocks
 // make less than two waves of them (1024 x 4096: 4.7 against 5.5 us) and at ragged edges,
 // whose guarded blocks take longer (4000 x 4004: 18.0 against 24.2 us).
+// X is no __restrict__ pointer: the kernel may start while its stream's previous kernel still writes X, so X's bytes
+// are not constant over the kernel and must not be read ahead of the dependency wait.
 template <bool VEC, int T>
 __global__ void __launch_bounds__(T, T == 256 ? 3 : 2)
-    quantize_kernel(const float* __restrict__ X, int64_t rows, int64_t cols, int64_t ldx, uint8_t* __restrict__ Q,
-                    int64_t ldq, float* __restrict__ scales, int64_t s_ld) {
+    quantize_kernel(const float* X, int64_t rows, int64_t cols, int64_t ldx, uint8_t* Q, int64_t ldq, float* scales,
+                    int64_t s_ld) {
   constexpr int kWarps = T / 32, kRows = 128 / kWarps;  // warps, rows per warp
   __shared__ float red[kWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
