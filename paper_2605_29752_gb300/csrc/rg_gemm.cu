@@ -105,7 +105,7 @@ struct GemmArgs {
   int32_t dp_tiles;         // stream-K: tiles run whole before the shared tail
   int32_t panel;            // tile order: column panels of this many tiles (pairs: tile columns)
   int32_t early;            // 1: A and B are static, so loads may start before the preceding grid completes
-  int32_t subs;             // accumulators a unit's K blocks are summed in, one after another (see accum_subs)
+  int32_t parts;            // parts that a unit's K blocks are summed in, or 0 (see accum_parts)
   int32_t whole;            // (pair) tiles run whole, the rest as two half-width units each (see tail_tiles)
   float* ws;                // split-K partials [split][tile][BM][BN]
   int32_t* tickets;         // [tile][4], zero between launches
@@ -113,6 +113,16 @@ struct GemmArgs {
   long long timeout;        // cycles per wait
   unsigned long long* trace;  // phase stamps [CTA][kTraceFields] (RG_PHASE_TIMERS builds), or null
 };
+
+// Whether the K blocks of a tile's units may be summed in several accumulators, one after another (TMEM columns of
+// an accumulator: BN, twice that for 256-row CTAs; four of them have to fit): the units of 1-CTA tiles, see
+// accum_parts, and grouped units that run all K splits of a tile in turn.
+__host__ __device__ constexpr bool multi_tile(int acc_cols) { return acc_cols <= 128; }
+// Whether those of its split-K units may be as well.
+__host__ __device__ constexpr bool multi_split_tile(int acc_cols) { return acc_cols <= 64; }
+
+// A part is at most kPartBlocks K blocks, on 128x64 summed in two halves beyond kAccBlocks.
+constexpr int kPartBlocks = 16, kAccBlocks = 12;
 
 // CTAS = 2: one CTA of a cta_group::2 pair (BM = 128 rows of its own, BN / 2
 // columns of B in its shared memory, M = 256 per MMA instruction).
@@ -126,14 +136,18 @@ struct KCfg {
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;  // one K block: A, then B
   static constexpr int HALVES = BM / 128;
   static constexpr int ACC_COLS = HALVES * BN;
-  static constexpr int NBUF = (2 * ACC_COLS <= 512) ? 2 : 1;
+  // Accumulators in TMEM: two where they fit, so that a tile's epilogue overlaps the next tile's MMAs; four where
+  // a unit may be summed in several (the sum so far, a part's two halves, and one that the MMAs fill).
+  static constexpr int NBUF = multi_tile(ACC_COLS) ? 4 : 2 * ACC_COLS <= 512 ? 2 : 1;
+  // Whether parts of more than kAccBlocks K blocks are summed in two halves (128x64)
+  static constexpr bool HALVED = ACC_COLS <= 64;
   static constexpr int USED_COLS = NBUF * ACC_COLS;
   static constexpr int TMEM_COLS = USED_COLS <= 32 ? 32 : USED_COLS <= 64 ? 64 : USED_COLS <= 128 ? 128
                                    : USED_COLS <= 256 ? 256 : 512;
   static constexpr int STAGING_OFF = STAGES * STAGE_BYTES;
   static constexpr int BAR_OFF = STAGING_OFF + 4 * kStagingPerWarp;
   static constexpr int SMEM_BYTES = 1024 + BAR_OFF + 256;
-  static_assert((2 * STAGES + 9) * 8 <= 256, "barrier block");
+  static_assert((2 * STAGES + 2 * NBUF + 5) * 8 <= 256, "barrier block");
   static constexpr uint32_t IDESC = instr_desc(1, 1, 0, 1, 128 * CTAS, BN);
   // Tiles whose columns can be halved in whole 64-column boxes per CTA (tail tiles).
   static constexpr bool HALVABLE = BN % (128 * CTAS) == 0;
@@ -215,14 +229,6 @@ __device__ __forceinline__ void store_block(const CUtensorMap* tmC, const float 
   sbuf ^= 1;
 }
 
-// Whether a tile's grouped units may run all K splits of a problem in turn: its epilogue threads
-// then hold one FP32 sum per accumulator column (TMEM columns: BN, twice that for 256-row CTAs).
-__host__ __device__ constexpr bool serial_tile(int acc_cols) { return acc_cols <= 128; }
-// Whether its units may sum their K blocks in several accumulators in turn (1-CTA tiles).
-__host__ __device__ constexpr bool segment_tile(int acc_cols) { return acc_cols <= 128; }
-// Whether its split-K units may as well.
-__host__ __device__ constexpr bool segment_split_tile(int acc_cols) { return acc_cols <= 64; }
-
 // One work unit: which output tile of which problem, which K blocks, and where
 // its operands and output live.
 struct Unit {
@@ -240,15 +246,17 @@ struct Unit {
   int tk0 = 0;       // first ticket of the problem (grouped launches)
   bool half = false; // the unit is half of its tile's columns (tail tiles),
   int noff = 0;      // the left (0) or the right (1) one
-  // Accumulators the unit's K blocks are summed in, one after another: all K splits of the tile (grouped launches), or
-  // `subs` equal parts; one of the two is 1.
-  int segs = 1, subs = 1;
+  // How the unit's K blocks are summed: those of all K splits of the tile, one after another (segs > 1: grouped
+  // launches), of each in `parts` parts (see accum_parts; 0: in one accumulator).
+  int segs = 1, parts = 0;
 };
 
-// K blocks of accumulator t of n of a unit that runs [kb0, kb1)  (32-bit: t < 64 and kb1 <= 2^24)
-__device__ __forceinline__ void sub_range(int kb0, int kb1, int n, int t, int& lo, int& hi) {
-  lo = kb0 + t * (kb1 - kb0) / n;
-  hi = kb0 + (t + 1) * (kb1 - kb0) / n;
+// K blocks of part t of n (a power of two) of a unit that runs [kb0, kb1)
+__device__ __forceinline__ void part_range(int kb0, int kb1, int n, int t, int& lo, int& hi) {
+  const int shift = 31 - __clz(n);
+  const int64_t len = kb1 - kb0;
+  lo = kb0 + static_cast<int>(t * len >> shift);
+  hi = kb0 + static_cast<int>((t + 1) * len >> shift);
 }
 
 // Tile order: the tile grid is cut into column panels `panel` tiles wide and
@@ -309,7 +317,7 @@ struct SingleSched {
   const CUtensorMap* w;
   int tiles_m, tiles_n, splits, kblocks, M, N, beta;
   int whole = 0;
-  int subs = 1;
+  int parts = 0;
   int panel = 1 << 30;
   __device__ __forceinline__ void prefetch() const {
     prefetch_tmap(a);
@@ -332,7 +340,7 @@ struct SingleSched {
       x.half = u >= whole;
       x.noff = h & 1;
     }
-    x.subs = subs;
+    x.parts = parts;
     return x;
   }
 };
@@ -574,7 +582,7 @@ struct alignas(128) GroupItem {
   int32_t tiles_n, kblocks, unit_start, splits;
   int32_t ws_row0, tk0;
   int32_t segs;  // K splits one unit runs in turn (splits is then 1), or 1
-  int32_t subs;  // accumulators of a split
+  int32_t parts;  // parts of a split, or 0
 };
 struct alignas(128) GroupHeader {
   int32_t n_items;
@@ -605,7 +613,7 @@ struct GroupSched {
   int rank = 0, cid = 0, ncl = 1;
   // the calling warp's current item and its sizes (unit() is called by whole warps, in ascending order)
   mutable int cur = 0, loaded = -1;
-  mutable int4 d0, d1, d2;  // {M, N, beta, tiles_m}, {tiles_n, kblocks, unit_start, splits}, {ws_row0, tk0, segs, subs}
+  mutable int4 d0, d1, d2;  // {M, N, beta, tiles_m}, {tiles_n, kblocks, unit_start, splits}, {ws_row0, tk0, segs, parts}
   __device__ __forceinline__ void prefetch() const {}
   __device__ __forceinline__ void init() {
     n_items = h->n_items;
@@ -686,7 +694,7 @@ struct GroupSched {
     x.ws_row0 = d2.x;
     x.tk0 = d2.y;
     x.segs = d2.z;
-    x.subs = d2.w;
+    x.parts = d2.w;
     return x;
   }
 };
@@ -708,12 +716,11 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
   constexpr bool P2 = Sched::k2Sm;  // one CTA of a cta_group::2 pair
   constexpr bool CS = IsClusterSplit<Sched>::value;  // one K slice of a cluster split-K tile
   using C = KCfg<BM, BN, STAGES, P2 ? 2 : 1>;
-  // units may sum several accumulators in turn (a thread then holds its sums of the whole tile in registers)
-  constexpr bool SERIAL = Sched::kMapsInGlobal ? (P2 ? serial_tile(C::ACC_COLS) : segment_tile(C::ACC_COLS))
-                          : IsSingle<Sched>::value && !CS && !Sched::kMemOnly
-                              ? (Sched::kSplit ? segment_split_tile(C::ACC_COLS) : segment_tile(C::ACC_COLS))
-                              : false;
-  constexpr bool SUBS_SPLIT = SERIAL && Sched::kSplit && !P2 && segment_split_tile(C::ACC_COLS);
+  // units may be summed in several accumulators
+  constexpr bool MULTI = Sched::kMapsInGlobal ? multi_tile(C::ACC_COLS)
+                         : IsSingle<Sched>::value && !CS && !Sched::kMemOnly
+                             ? (Sched::kSplit ? multi_split_tile(C::ACC_COLS) : multi_tile(C::ACC_COLS))
+                             : false;
   constexpr bool TAIL = HasTail<Sched>::value;  // units may be halves of their tile's columns
   static_assert(!TAIL || C::HALVABLE, "tail tiles");
   extern __shared__ uint8_t smem_raw[];
@@ -725,14 +732,15 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
   auto full_bar = [&](int i) { return bar0 + 8u * i; };
   auto empty_bar = [&](int i) { return bar0 + 8u * (STAGES + i); };
   auto tfull_bar = [&](int b) { return bar0 + 8u * (2 * STAGES + b); };
-  auto tempty_bar = [&](int b) { return bar0 + 8u * (2 * STAGES + 2 + b); };
-  const uint32_t drain_bar = bar0 + 8u * (2 * STAGES + 4);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 5);
+  auto tempty_bar = [&](int b) { return bar0 + 8u * (2 * STAGES + C::NBUF + b); };
+  constexpr int kBars = 2 * STAGES + 2 * C::NBUF;  // of stages and accumulators
+  const uint32_t drain_bar = bar0 + 8u * kBars;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kBars + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   // cluster split-K: the other CTAs' operand rings are free / their blocks for this CTA have landed
-  const uint32_t go_bar = bar0 + 8u * (2 * STAGES + 6);
-  const uint32_t recv_bar = bar0 + 8u * (2 * STAGES + 7);
-  const uint32_t ready_bar = bar0 + 8u * (2 * STAGES + 8);  // this CTA's four epilogue warps saw the sum final
+  const uint32_t go_bar = bar0 + 8u * (kBars + 2);
+  const uint32_t recv_bar = bar0 + 8u * (kBars + 3);
+  const uint32_t ready_bar = bar0 + 8u * (kBars + 4);  // this CTA's four epilogue warps saw the sum final
   int never = 0;
   volatile int* no_abort = &never;
 
@@ -745,7 +753,7 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
       mbar_init(full_bar(i), 1);
       mbar_init(empty_bar(i), 1);
     }
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < C::NBUF; ++b) {
       mbar_init(tfull_bar(b), 1);
       // pair: the even CTA's accumulator is free once both CTAs' epilogue warps drained it
       mbar_init(tempty_bar(b), P2 ? 8 : 4);
@@ -868,22 +876,32 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
     if (stall) ok = mbar_wait_warp(drain_bar, 0, timeout, abort_flag);
     // a pair's odd CTA issues nothing: the even CTA's MMAs read and write both
     const int issue_units = (!P2 || sched.rank == 0) ? nunits : 0;
-    // the K range and segments of the next unit, looked up while the current one's MMAs run
-    int kb0n = 0, kb1n = 0, segsn = 1, subsn = 1;
+    // the K range and parts of the next unit, looked up while the current one's MMAs run
+    int kb0n = 0, kb1n = 0, nparts = 1;
+    bool halve = false;
     uint32_t idesc = C::IDESC;
     if (issue_units > 0) {
       const Unit w = sched.unit(0);
       kb0n = w.kb0;
       kb1n = w.kb1;
-      segsn = w.segs;
-      subsn = w.subs;
+      nparts = w.segs * max(w.parts, 1);
+      halve = w.parts > 0;
       if (TAIL && w.half) idesc = C::IDESC_HALF;
     }
-    int seg = 0;
+    int part = 0;
+    bool second = false;  // the accumulator is the second half of its part
     for (int i = 0; ok && i < issue_units;) {
-      // the unit's K blocks, or those of its accumulator `seg`
+      // the K blocks of the unit, or of one of its accumulators
       int kb0 = kb0n, kb1 = kb1n;
-      if (SERIAL && segsn * subsn > 1) sub_range(kb0n, kb1n, segsn * subsn, seg, kb0, kb1);
+      bool more = false;  // the accumulator is the first half of its part
+      if constexpr (MULTI) {
+        if (nparts > 1) part_range(kb0n, kb1n, nparts, part, kb0, kb1);
+        if (C::HALVED && halve && kb1 - kb0 > kAccBlocks) {
+          const int mid = kb0 + (kb1 - kb0) / 2;
+          more = !second;
+          if (second) kb0 = mid; else kb1 = mid;
+        }
+      }
       ok = mbar_wait_warp(tempty_bar(acc), aph ^ 1u, timeout, abort_flag);
       if (!ok) break;
       tc_fence_after();
@@ -891,7 +909,7 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
       for (int kb = kb0; kb < kb1; ++kb) {
         ok = mbar_wait_warp(full_bar(stage), ph, timeout, abort_flag);
         if (!ok) break;
-        if (i == 0 && kb == kb0 && lane == 0) RG_STAMP(4);
+        if (i == 0 && part == 0 && !second && kb == kb0 && lane == 0) RG_STAMP(4);
         tc_fence_after();
         if constexpr (Sched::kMemOnly) {
           if (lane == 0) mbar_arrive(empty_bar(stage));  // no MMA reads the stage: it is free once its bytes have landed
@@ -925,14 +943,17 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
         acc = 0;
         aph ^= 1u;
       }
-      if (SERIAL && ++seg < segsn * subsn) continue;
-      seg = 0;
+      if constexpr (MULTI) {
+        second = more;
+        if (more || ++part < nparts) continue;
+        part = 0;
+      }
       if (++i < issue_units) {
         const Unit w = sched.unit(i);
         kb0n = w.kb0;
         kb1n = w.kb1;
-        segsn = w.segs;
-        subsn = w.subs;
+        nparts = w.segs * max(w.parts, 1);
+        halve = w.parts > 0;
         if (TAIL && w.half) idesc = C::IDESC_HALF;
       } else if (lane == 0) {
         RG_STAMP(5);
@@ -962,46 +983,84 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
     int acc = 0, sbuf = 0;
     uint32_t aph = 0;
     bool ok = true;
-    // The sum of the unit's accumulators, the first of which is ready; the last is left to be released.
-    auto sum_accumulators = [&](const Unit& w, int& acc, uint32_t& aph, float (&sum)[C::ACC_COLS / 32][32]) {
-      // -0 is the sum's neutral element (-0 + x = x, also for x = -0)
+    const uint32_t tq = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
+    auto acc_at = [&](int b) { return tq + static_cast<uint32_t>(b * C::ACC_COLS); };
+    auto release = [&](int b) {  // after tc_fence_before and __syncwarp
+      if (lane == 0) {
+        if constexpr (P2)
+          mbar_arrive_cluster(mapa_shared(tempty_bar(b), 0));  // the even CTA's MMA reuses it
+        else
+          mbar_arrive(tempty_bar(b));
+      }
+    };
+    // The result of a unit, or of its parts so far, is that of accumulator `acc` (0 where it has no K blocks: !some),
+    // added to that of its part's first half, `lower`, added to the sum of the parts before it, `before` (where they are
+    // not -1).
+    int lower = -1, before = -1;
+    bool some = true;
+    auto load_result = [&](int col, float (&v)[32]) {
+      uint32_t r[32], x[32];
+      tmem_ld_32x32b_x32(acc_at(acc) + col, r);
+      if (C::HALVED && lower >= 0) {
+        tmem_ld_32x32b_x32(acc_at(lower) + col, x);
+        tmem_ld_wait_for(r);
+        tmem_ld_wait_for(x);
 #pragma unroll
-      for (int c = 0; c < C::ACC_COLS / 32; ++c)
+        for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(x[e]) + __uint_as_float(r[e]);
+      } else {
+        tmem_ld_wait_for(r);
 #pragma unroll
-        for (int e = 0; e < 32; ++e) sum[c][e] = -0.f;
-      const int n = w.segs * w.subs;
+        for (int e = 0; e < 32; ++e) v[e] = some ? __uint_as_float(r[e]) : 0.f;
+      }
+      if (before >= 0) {
+        tmem_ld_32x32b_x32(acc_at(before) + col, x);
+        tmem_ld_wait_for(x);
+#pragma unroll
+        for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(x[e]) + v[e];
+      }
+    };
+    // Waits for a unit's accumulators, the first of which is ready, and sums its parts but the last (which is added as
+    // the result is stored) in the place of their last accumulators, while the MMAs of later ones run.
+    // (With the sums in registers, a thread holding its row of the tile, the grouped kernels of 128 accumulator columns
+    // spilled 540-596 bytes, against 48-56 so; and 512 x 512 x 4096 on 128x128 took 13.3 us, against 12.8.)
+    auto gather = [&](const Unit& w) {
+      auto next = [&] {
+        if (++acc == C::NBUF) {
+          acc = 0;
+          aph ^= 1u;
+        }
+        if (!mbar_wait_warp(tfull_bar(acc), aph, timeout, abort_flag)) return false;
+        tc_fence_after();
+        return true;
+      };
+      const int n = w.segs * max(w.parts, 1);
 #pragma unroll 1
-      for (int seg = 0; seg < n; ++seg) {
-        if (seg > 0) {
+      for (int part = 0;; ++part) {
+        int lo = w.kb0, hi = w.kb1;
+        if (n > 1) part_range(w.kb0, w.kb1, n, part, lo, hi);
+        some = hi > lo;
+        lower = -1;
+        if (C::HALVED && w.parts > 0 && hi - lo > kAccBlocks) {
+          lower = acc;
+          if (!next()) return false;
+        }
+        if (part == n - 1) return true;
+        if (lower >= 0 || before >= 0 || !some) {
+#pragma unroll 1
+          for (int c = 0; c < C::ACC_COLS / 32; ++c) {
+            float v[32];
+            load_result(c * 32, v);
+            tmem_st_32x32b_x32(acc_at(acc) + c * 32, v);
+          }
+          tmem_st_wait();
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) {
-            if constexpr (P2)
-              mbar_arrive_cluster(mapa_shared(tempty_bar(acc), 0));
-            else
-              mbar_arrive(tempty_bar(acc));
-          }
-          if (++acc == C::NBUF) {
-            acc = 0;
-            aph ^= 1u;
-          }
-          if (!mbar_wait_warp(tfull_bar(acc), aph, timeout, abort_flag)) return false;
-          tc_fence_after();
+          if (lower >= 0) release(lower);
+          if (before >= 0) release(before);
         }
-        int lo, hi;
-        sub_range(w.kb0, w.kb1, n, seg, lo, hi);
-        const bool some = hi > lo;  // the accumulator has K blocks
-        const uint32_t t = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * C::ACC_COLS);
-#pragma unroll
-        for (int c = 0; c < C::ACC_COLS / 32; ++c) {
-          uint32_t v[32];
-          tmem_ld_32x32b_x32(t + c * 32, v);
-          tmem_ld_wait_for(v);
-#pragma unroll
-          for (int e = 0; e < 32; ++e) sum[c][e] += some ? __uint_as_float(v[e]) : 0.f;
-        }
+        before = acc;
+        if (!next()) return false;
       }
-      return true;
     };
     for (int i = 0; i < nunits; ++i) {
       const Unit w = sched.unit(i);
@@ -1011,7 +1070,15 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
       if (i == 0 && warp == 2 && lane == 0) RG_STAMP(6);
       tc_fence_after();
       const bool have = kb1 > kb0;
-      uint32_t tacc = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * C::ACC_COLS);
+      if constexpr (MULTI) {
+        lower = before = -1;
+        some = have;
+        if (w.segs > 1 || w.parts > 1 || (C::HALVED && w.parts == 1 && kb1 - kb0 > kAccBlocks)) {
+          ok = gather(w);
+          if (!ok) break;
+        }
+      }
+      const uint32_t tacc = acc_at(acc);
       if constexpr (CS) {
         // Split-K inside the cluster, through distributed shared memory.  Block b = q kPerWarp + j
         // (32 x 32, j = h kCols + c) of the tile is reduced by CTA b % S; the other CTAs write their
@@ -1081,54 +1148,47 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
           store_block(w.c, sum, tm * BM + (j / kCols) * 128 + q * 32, tn * BN + (j % kCols) * 32, w.M, w.N, w.beta,
                       stg0, sbuf, lane);
         }
-      } else if (SERIAL && (w.segs > 1 || (w.subs > 1 && (!SUBS_SPLIT || w.splits == 1)))) {
-        // Several accumulators, one after another, summed in registers: all K splits of the tile (their sum in the
-        // order 0..S-1, as the workspace path's last arriver forms it, without the partials' round
-        // trip through memory; publishing, waiting for and re-reading a split's partial takes an
-        // epilogue warp 3-6 us: 8 problems of 512 x 576 x 1024 on 128x64, S = 4, 59.5 us; without
-        // a split 18.5), or the unit's `subs` parts.
-        if constexpr (SERIAL) {
-          float sum[C::ACC_COLS / 32][32];
-          ok = sum_accumulators(w, acc, aph, sum);
-          if (!ok) break;
-#pragma unroll
-          for (int c = 0; c < C::ACC_COLS / 32; ++c)
-            store_block(w.c, sum[c], tm * BM + (c * 32 / BN) * 128 + q * 32, tn * BN + c * 32 % BN, w.M, w.N, w.beta, stg0,
-                        sbuf, lane);
-        }
       } else if (!Sched::kSplit || w.splits == 1) {
         const int cols = TAIL && w.half ? BN / 2 : BN, col0 = tn * BN + (TAIL && w.half ? w.noff * (BN / 2) : 0);
+        if (MULTI && (lower >= 0 || before >= 0)) {
 #pragma unroll 1
-        for (int h = 0; h < C::HALVES; ++h)
+          for (int h = 0; h < C::HALVES; ++h)
 #pragma unroll 1
-          for (int c = 0; c < cols / 32; ++c) {
-            float v[32];
-            load_acc(tacc + h * BN + c * 32, have, v);
-            store_block(w.c, v, tm * BM + h * 128 + q * 32, col0 + c * 32, w.M, w.N, w.beta, stg0, sbuf, lane);
-          }
+            for (int c = 0; c < cols / 32; ++c) {
+              float v[32];
+              load_result(h * BN + c * 32, v);
+              store_block(w.c, v, tm * BM + h * 128 + q * 32, col0 + c * 32, w.M, w.N, w.beta, stg0, sbuf, lane);
+            }
+        } else {
+#pragma unroll 1
+          for (int h = 0; h < C::HALVES; ++h)
+#pragma unroll 1
+            for (int c = 0; c < cols / 32; ++c) {
+              float v[32];
+              load_acc(tacc + h * BN + c * 32, have, v);
+              store_block(w.c, v, tm * BM + h * 128 + q * 32, col0 + c * 32, w.M, w.N, w.beta, stg0, sbuf, lane);
+            }
+        }
       } else if constexpr (Sched::kSplit) {
         // Split-K.  Publish this split's FP32 partial tile: TMEM -> swizzled staging ->
         // TMA store into the workspace (rows (s * ntiles + tile) * BM ..), then wait
         // for the stores, fence them against the generic proxy and take the ticket
         // of this (tile, warp) row block with an acquire-release atomic.
         const int wrow = w.ws_row0 + (s * ntiles + tile) * BM;
-        if constexpr (SUBS_SPLIT) {
-          if (w.subs > 1) {  // the split's sum takes the place of its last accumulator
-            float sum[C::ACC_COLS / 32][32];
-            ok = sum_accumulators(w, acc, aph, sum);
-            if (!ok) break;
-            tacc = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * C::ACC_COLS);
-#pragma unroll
-            for (int c = 0; c < C::ACC_COLS / 32; ++c) tmem_st_32x32b_x32(tacc + c * 32, sum[c]);
-            tmem_st_wait();
-          }
-        }
+        // A warp's two staging buffers still hold the partial of a 128x64 tile's two blocks when its stores are done, in
+        // the layout that the sum below needs; that of a larger tile is read from TMEM again.
+        constexpr bool kOwnStaged = C::HALVES * (BN / 32) == 2;
+        static_assert(kOwnStaged || !MULTI || Sched::kMapsInGlobal, "a split's result has to be one accumulator");
+        const int sbuf0 = sbuf;
 #pragma unroll 1
         for (int h = 0; h < C::HALVES; ++h)
 #pragma unroll 1
           for (int c = 0; c < BN / 32; ++c) {
             float v[32];
-            load_acc(tacc + h * BN + c * 32, have, v);
+            if (MULTI && (lower >= 0 || before >= 0))
+              load_result(h * BN + c * 32, v);
+            else
+              load_acc(tacc + h * BN + c * 32, have, v);
             store_block(w.w, v, wrow + h * 128 + q * 32, c * 32, INT_MAX, INT_MAX, 0, stg0, sbuf, lane);
           }
         if (lane == 0) {
@@ -1154,8 +1214,10 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
           // The last arriver sums the S partials of each 32 x 32 block in the fixed
           // order 0..S-1.  Lane l holds block rows 4j + l/8 (j = 0..7), columns
           // 4(l%8)..4(l%8)+3, so each warp load reads four whole 128-byte rows;
-          // partials are loaded kBatch at a time.  Its own partial (still in TMEM,
-          // one row per lane) is brought into that layout through the staging buffer.
+          // partials are loaded kBatch at a time.  Its own partial, one row per lane, is
+          // brought into that layout through the staging buffers: it is still there (two
+          // blocks; not reading it again, 512 x 512 x 1024 on 128x64 with S = 2 went from
+          // 7.0 to 6.6 us) or comes from TMEM once more.
           constexpr int kBatch = 3;
           const int rsub = lane >> 3, g = lane & 7;
           if (w.splits == 2) {
@@ -1187,16 +1249,18 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
                 for (int j = 0; j < 8; ++j)
                   nxt[j] = __ldcg(reinterpret_cast<const float4*>(src + static_cast<size_t>(4 * j + rsub) * BN));
               }
-              float own[32];
-              load_acc(tacc + h * BN + c * 32, have, own);
-              if (lane == 0) bulk_wait_read<1>();
-              __syncwarp();
-              const uint32_t buf = stg0 + sbuf * 4096;
+              const uint32_t buf = stg0 + (kOwnStaged ? sbuf0 ^ ch : sbuf) * 4096;
+              if constexpr (!kOwnStaged) {
+                float own[32];
+                load_acc(tacc + h * BN + c * 32, have, own);
+                if (lane == 0) bulk_wait_read<1>();
+                __syncwarp();
 #pragma unroll
-              for (int j = 0; j < 8; ++j)
-                st_shared_v4(buf + lane * 128 + ((j ^ (lane & 7)) << 4), own[4 * j], own[4 * j + 1], own[4 * j + 2],
-                             own[4 * j + 3]);
-              __syncwarp();
+                for (int j = 0; j < 8; ++j)
+                  st_shared_v4(buf + lane * 128 + ((j ^ (lane & 7)) << 4), own[4 * j], own[4 * j + 1], own[4 * j + 2],
+                               own[4 * j + 3]);
+                __syncwarp();
+              }
               float4 sum[8];
 #pragma unroll
               for (int j = 0; j < 8; ++j) {
@@ -1229,16 +1293,18 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
           for (int h = 0; h < C::HALVES; ++h)
 #pragma unroll 1
             for (int c = 0; c < BN / 32; ++c) {
-              float own[32];
-              load_acc(tacc + h * BN + c * 32, have, own);
-              if (lane == 0) bulk_wait_read<1>();
-              __syncwarp();
-              const uint32_t buf = stg0 + sbuf * 4096;
+              const uint32_t buf = stg0 + (kOwnStaged ? sbuf0 ^ c : sbuf) * 4096;
+              if constexpr (!kOwnStaged) {
+                float own[32];
+                load_acc(tacc + h * BN + c * 32, have, own);
+                if (lane == 0) bulk_wait_read<1>();
+                __syncwarp();
 #pragma unroll
-              for (int j = 0; j < 8; ++j)
-                st_shared_v4(buf + lane * 128 + ((j ^ (lane & 7)) << 4), own[4 * j], own[4 * j + 1], own[4 * j + 2],
-                             own[4 * j + 3]);
-              __syncwarp();
+                for (int j = 0; j < 8; ++j)
+                  st_shared_v4(buf + lane * 128 + ((j ^ (lane & 7)) << 4), own[4 * j], own[4 * j + 1], own[4 * j + 2],
+                               own[4 * j + 3]);
+                __syncwarp();
+              }
               float4 o[8], sum[8];
 #pragma unroll
               for (int j = 0; j < 8; ++j) {
@@ -1303,12 +1369,11 @@ __device__ __forceinline__ void gemm_body(Sched& sched, float* ws, int32_t* tick
 #endif
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) {
-        if constexpr (P2)
-          mbar_arrive_cluster(mapa_shared(tempty_bar(acc), 0));  // the even CTA's MMA reuses it
-        else
-          mbar_arrive(tempty_bar(acc));
+      if constexpr (MULTI) {
+        if (lower >= 0) release(lower);
+        if (before >= 0) release(before);
       }
+      release(acc);
       if (++acc == C::NBUF) {
         acc = 0;
         aph ^= 1u;
@@ -1354,7 +1419,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   SingleSched<SPLIT, !SPLIT && KCfg<BM, BN, STAGES>::HALVABLE> sched{
       &tmA, &tmB, &tmC, &tmW, args.tiles_m, args.tiles_n, args.splits, args.kblocks, args.M, args.N, args.beta};
   sched.whole = args.whole;
-  sched.subs = args.subs;
+  sched.parts = args.parts;
   sched.panel = args.panel;
   gemm_body<BM, BN, STAGES>(sched, args.ws, args.tickets, args.err, args.timeout, args.stall, args.early, args.trace);
 }
@@ -1672,21 +1737,26 @@ static int64_t tail_tiles(int64_t tiles, int64_t p) {
   return tiles >= p && 2 * r <= p ? r : 0;
 }
 
-// The accumulators that a launch's units sum their K blocks in, one after another (1-CTA tiles of up to 128
-// accumulator columns; of 64 with split-K; fewer tiles than SMs, where split-K is an alternative).  An accumulator's
-// error grows with its K, about 1e-9 of the result per element, so the variant with the most splits has the closest
-// sums; with no more than 1024 of K to an accumulator the others are as close, and the epilogue adds a finished
-// accumulator while the MMAs fill the next.  Error (2-norm, relative) on 128x64: 512 x 1736 x 2864 2.7e-6 -> 7.9e-7,
-// 2176 x 384 x 2806 2.7e-6 -> 7.7e-7, and with S = 2 72 x 4096 x 4096 1.9e-6 -> 8.5e-7 (11.3 -> 11.9 us).
-static int32_t accum_subs(const rg_ctx* ctx, int32_t variant, int64_t rows, int64_t cols, int64_t depth) {
+// The parts that a launch's units sum their K blocks in: 1-CTA tiles of up to 128 accumulator columns (128x64, 128x128,
+// 256x64), of 64 with split-K; fewer tiles than SMs, where split-K is an alternative.  An accumulator's error grows with
+// its K, about 1e-9 of the result per element, so a plan that picks the fastest variant must not lose by it what split-K
+// would have kept.  The parts are as many as a split count (1, 2, 4, 8, 16, ..) and at most 1024 of K each; on 128x64,
+// the tile that a sweep takes S = 4 of for K beyond about 1800, those of more than 768 are summed in two halves.  The
+// epilogue sums finished parts while the MMAs fill the next ones.  Error (2-norm, relative) and time on 128x64, against
+// parts as few as 1024 of K allows, in registers: 512 x 512 x 2048 8.5e-7 -> 3.9e-7, 7.96 -> 7.35 us; 208 x 256 x 2560
+// 7.0e-7 -> 5.0e-7; with S = 2 128 x 4096 x 4096 8.5e-7 -> 4.0e-7, 10.9 -> 11.0 us.  One accumulator over all of K: 1.9e-6
+// at 2048.
+static int32_t accum_parts(const rg_ctx* ctx, int32_t variant, int64_t rows, int64_t cols, int64_t depth) {
   const TileKernel& tk = tile_kernel(variant_tile(variant));
   const int splits = variant_split(variant), acc_cols = tk.bm / 128 * tk.bn;
   if (variant_streamk(variant) || variant_2sm(variant) ||
-      !(splits > 1 ? segment_split_tile(acc_cols) : segment_tile(acc_cols)) ||
+      !(splits > 1 ? multi_split_tile(acc_cols) : multi_tile(acc_cols)) ||
       (rows + tk.bm - 1) / tk.bm * ((cols + tk.bn - 1) / tk.bn) >= ctx->sm_count)
-    return 1;
+    return 0;
   const int64_t kblocks = ((depth + kBK - 1) / kBK + splits - 1) / splits;
-  return static_cast<int32_t>(std::min<int64_t>((kblocks + 15) / 16, 64));
+  int32_t parts = 1;
+  while (static_cast<int64_t>(parts) * kPartBlocks < kblocks) parts *= 2;
+  return parts;
 }
 
 struct Launch {
@@ -1801,7 +1871,7 @@ static int prepare(rg_ctx* ctx, int64_t M, int64_t N, int64_t K, const void* A, 
   g.splits = sk ? static_cast<int32_t>(skg.tail_ctas) : splits;  // stream-K: CTAs sharing the tail tiles
   g.dp_tiles = sk ? static_cast<int32_t>(skg.dp_tiles) : 0;
   g.kblocks = static_cast<int32_t>(kblocks);
-  g.subs = accum_subs(ctx, variant, pm, pn, pk);
+  g.parts = accum_parts(ctx, variant, pm, pn, pk);
   g.whole = static_cast<int32_t>(tiles_m * tiles_n);
   if (splits == 1 && !sk && tk.bn % (two ? 256 : 128) == 0)
     g.whole -= static_cast<int32_t>(tail_tiles(tiles_m * tiles_n, two ? ctx->sm_count / 2 : ctx->sm_count));
@@ -1901,7 +1971,7 @@ static int plan_launches(rg_ctx* ctx, const rg_plan* plan, int64_t M, int64_t N,
     if (rc != RG_OK) return rc;
     if (part) {  // rows of a leaf: summed as the whole leaf's
       const int64_t rows = std::min(lf.m, M - lf.m0);
-      L.args.subs = accum_subs(ctx, lf.variant, lf.pm ? lf.pm : rows, lf.pn ? lf.pn : n, lf.pk ? lf.pk : k);
+      L.args.parts = accum_parts(ctx, lf.variant, lf.pm ? lf.pm : rows, lf.pn ? lf.pn : n, lf.pk ? lf.pk : k);
     }
     out.push_back(L);
   }
@@ -2836,7 +2906,7 @@ extern "C" int rg_gemm_grouped(rg_group* g, const rg_group_problem* probs, int32
   // The K splits of a tile as one unit, where that is no longer than a CTA's (cluster's) share of
   // the family's K blocks: splitting then only adds the partials' traffic, not parallelism.
   auto serial_splits = [&](const Prepared& q) {
-    return q.L.args.splits > 1 && q.L.args.subs == 1 && rg::serial_tile(rg::family_bn(q.family) * (cta_rows(q.family) / 128)) &&
+    return q.L.args.splits > 1 && q.L.args.parts <= 1 && rg::multi_tile(rg::family_bn(q.family) * (cta_rows(q.family) / 128)) &&
            q.L.args.kblocks * sharers(q.family) <= blocks[q.family];
   };
   for (const auto& q : prep) {  // partials and tickets of the other splits
@@ -2881,7 +2951,7 @@ extern "C" int rg_gemm_grouped(rg_group* g, const rg_group_problem* probs, int32
     it.unit_start = static_cast<int32_t>(list.units[f]);
     it.splits = splits;
     it.segs = serial ? a.splits : 1;
-    it.subs = a.subs;
+    it.parts = a.parts;
     it.ws_row0 = static_cast<int32_t>(my_rows > 0 ? row0 : 0);
     it.tk0 = static_cast<int32_t>(list.tickets);
     list.items[f].push_back(it);
