@@ -231,7 +231,16 @@ int rg_launch_count(const rg_ctx* ctx, int64_t* out);
  * 256x192 1-CTA tiles (not 256x256 with S = 8) runs as clusters of S CTAs that sum the
  * S partials through distributed shared memory; the other split variants sum
  * them through the context's workspace.  Both sum in the order 0..S-1, so the
- * two forms give the same bits. */
+ * two forms give the same bits.
+ * A result is the same on every call with the same arguments.  From one call to
+ * another a row keeps its bits with the variant, K and pk and, for the tiles that
+ * follow, with the launch's size: launches of fewer tiles (of pm x pn) than the
+ * GPU has SMs sum K in parts on the 1-CTA 128x64 tile (any S) and, with S = 1, on
+ * 128x128 and 256x64 -- as many parts of pk / S as a power of two gives at most
+ * 1024 of K each, on 128x64 those of more than 768 in two halves -- where larger
+ * launches, and the other tiles, sum K in one accumulator.  So a row computed in
+ * a small launch may differ in its last bits from the same row in a large one,
+ * or with other padded extents; the parts are the closer to the exact sum. */
 int rg_gemm(rg_ctx* ctx, int64_t M, int64_t N, int64_t K,
             const void* A, int64_t lda, const void* B, int64_t ldb,
             float* C, int64_t ldc, int32_t variant, int32_t beta,
