@@ -504,21 +504,13 @@ __device__ __forceinline__ void fp8_body(const CUtensorMap& tmA, const CUtensorM
         }
         continue;
       }
-      // One store loop for both cases: C itself (S = 1) or this split's slot of
-      // the workspace (S > 1), which the last arriving split then reduces.
-      const bool direct = !SPLIT || S == 1;
-      const CUtensorMap* dst = direct ? &tmC : &tmW;
-      const int drow = direct ? row0 : (s * ntiles + tile) * BM + q * 32;
-      const int dcol = direct ? tn * BN : 0;
-      const bool dadd = direct && args.beta != 0;
+      if constexpr (SPLIT) {
+      // Split-K: store the partial to this split's slot of the workspace, wait for
+      // the stores, fence them against the generic proxy and take the (tile, warp)
+      // ticket.
 #pragma unroll
       for (int c = 0; c < C::HALF / 32; ++c)
-        if (!direct || (row0 < args.M && dcol + hc * C::HALF + c * 32 < args.N))
-          put_block<C::NSTG>(dst, r + c * 32, drow, dcol + hc * C::HALF + c * 32, dadd, stg0, sbuf, lane);
-      if (direct) continue;
-      if constexpr (SPLIT) {
-      // Split-K: wait for this split's stores, fence them against the generic
-      // proxy and take the (tile, warp) ticket.
+        put_block<C::NSTG>(&tmW, r + c * 32, (s * ntiles + tile) * BM + q * 32, hc * C::HALF + c * 32, false, stg0, sbuf, lane);
       if (lane == 0) {
         bulk_wait<0>();
         fence_proxy_async_global();

@@ -48,7 +48,6 @@
 #include <mutex>
 #include <string>
 #include <type_traits>
-#include <type_traits>
 #include <vector>
 
 #include "ptx.cuh"
