@@ -331,7 +331,8 @@ int rg_surface_stats(const rg_grid* grid, const int64_t* t_ns, double* tflops_ou
  * over all SMs whose work units are the concatenation of its problems'
  * (tile, K split) units, longest first.  Where a family's tiles fill the chip, its
  * split problems run all K splits of a tile in turn on one CTA (pair) instead (the
- * 128x64, 128x128, 256x64 tiles and the 256x128 pairs).  Each problem has its own
+ * 128x64, 128x128, 256x64 tiles and the 256x128 pairs; not a 128x64 problem whose
+ * splits are summed in several parts each, see rg_gemm).  Each problem has its own
  * sizes, operands, leading dimensions, beta and padded launch extents (pm, pn, pk
  * as in rg_gemm; 0 = no padding).  The split-K partials and tickets live in a
  * workspace the group owns (workspace_bytes, at least 1 MiB); when the problems

@@ -8,15 +8,14 @@
 //              (64 x BN, N-major, 128B swizzle, 64-column boxes) into an
 //              mbarrier-guarded ring of STAGES shared-memory stages, one K block each.
 //   warp 1     allocates TMEM; one lane issues tcgen05.mma (M = 128, N = BN,
-//              K = 16) into a TMEM accumulator, double-buffered when it fits,
-//              and commits stage releases / accumulator-full to mbarriers.
+//              K = 16) into one of the TMEM accumulators (two where they fit, four of
+//              up to 128 columns), and commits stage releases / accumulator-full to
+//              mbarriers.
 //   Both warps step through their loops converged: all lanes test the barriers, a
 //   vote makes the outcome uniform, and the loads, MMAs and commits are predicated
-//   instructions of one elected lane.  tcgen05.mma and the TMA instructions take
-//   their operands from uniform registers; in code that one lane runs by itself
-//   every operand is first moved there, which made each MMA cost about 95 cycles of
-//   issue whatever its size (N = 64 at M = 128 needs 48, bound by its operand reads;
-//   N = 128 needs 64, N = 256 needs 128).  K blocks of 64, cycles each at 2.07 GHz,
+//   instructions of one elected lane.  With one lane in the loop by itself an MMA took
+//   about 95 cycles of issue whatever its size (N = 64 at M = 128 needs 48, N = 128 64,
+//   N = 256 128).  K blocks of 64, cycles each at 2.07 GHz,
 //   512 x 512 x 4096, before and after: 128x64 390 -> 205, 128x128 385 -> 275,
 //   256x64 (two MMAs per K step) 680 -> 395, the 256x128 pair 420 -> 275,
 //   128x192 510 -> 405; 128x256 and the 256x256 tiles were at the MMA rate.
@@ -1726,9 +1725,10 @@ static int make_map(CUtensorMap* m, CUtensorMapDataType dt, const void* base, ui
 }
 
 // Tiles of the last, partial wave that run as two units of half the columns each: those r tiles of T = w P + r
-// (P CTAs, or clusters for pair tiles) for which the chip has room, w >= 1 and 2 r <= P; else 0.  The halves take
-// about half a tile's time (their MMAs have half the columns) on SMs that the last wave would leave idle; every
-// output is summed over K in the same order either way.  Tiles of 128 and 256 columns (pairs: 256).
+// (P CTAs, or clusters for pair tiles) for which the chip has room, w >= 1 and 2 r <= P; else 0.  The halves run on
+// SMs that the last wave would leave idle, and store half the columns each; a K block of one takes half a tile's time
+// for 256 columns and about three quarters for 128 (205 of 275 cycles: MMAs of 64 columns are not at the full rate).
+// Every output is summed over K in the same order either way.  Tiles of 128 and 256 columns (pairs: 256).
 // 4096^3 on 256x256 pairs, r/P = 28/76: 80.1 -> 74.0 us; 4096 x 1280 x 4096, 4/76: 40.8 -> 32.6 (stream-K 40.4);
 // 2560 x 1024 x 2048 on 128x128, 8/152: 15.6 -> 13.7.
 static int64_t tail_tiles(int64_t tiles, int64_t p) {

@@ -482,7 +482,7 @@ extern "C" int rg_serve(rg_ctx* ctx, const rg_plan* plan, const rg_serve_opts* o
 // pass on: submissions it has been told of, results that have come in since.  (A
 // step that scanned every request ever submitted, under the mutex, and woke every
 // waiter grew with the server's age: a burst of 24 mixed requests took 240 us at first
-// and 622 after 1,500 such bursts; now 165 at any age.)
+// and 622 after 1,500 such bursts; now 166-179 at any age, by the box.)
 struct rg_server {
   rg_ctx* ctx = nullptr;
   Engine* eng = nullptr;
