@@ -5,14 +5,17 @@ the smoothed stack (autotuned best-of tiles and split factors + the DP
 padding/splitting plan, O(1) lookup, fused execution), on one GB300.
 
 Setup (not timed, "offline once per hardware/software stack"): the autotune
-sweep times all 38 kernel variants (6 tiles x {split-K 1/2/4/8, stream-K}, and
-the two 256-row tiles as tcgen05 cta_group::2 pairs with split-K 1/2/4/8) on
-every cell, with the library's pruning, and builds the plan tables.  One timed step re-measures, for every cell, the
-plain fixed 128x128 tile and the smoothed plan with the paper's protocol (one
-warm-up launch, then the mean of 5 back-to-back launches between CUDA events),
-then computes both surfaces' mean and roughness in the library.
+sweep times all 55 kernel variants (8 tiles x {split-K 1/2/4/8, stream-K}, and
+three of them as tcgen05 cta_group::2 pairs with split-K 1/2/4/8 and stream-K)
+on every cell, with the library's pruning, and builds the plan tables.  One
+timed step re-measures, for every cell, the plain fixed 128x128 tile and the
+smoothed plan with the paper's protocol (one warm-up launch, then the mean of 5
+back-to-back launches between CUDA events), then computes both surfaces' mean
+and roughness in the library.
 
-Prints one JSON line (rank 0).  --impl reference times the CPU oracle instead.
+Prints one JSON line (rank 0) of the results that name the run; the whole record
+(the ladder, the other surfaces, the studies) goes to standard error as one JSON
+line, and to --out.  --impl reference times the CPU oracle instead.
 """
 from __future__ import annotations
 
@@ -45,7 +48,7 @@ def parse():
     p.add_argument("--impl", default="ours", choices=["ours", "reference"])
     p.add_argument("--count", type=int, default=COUNT, help="grid points per axis (32 = the full grid)")
     p.add_argument("--no-extras", action="store_true", help="skip the ladder / cross-tile / e2e / CPU sections")
-    p.add_argument("--out", default=None, help="also write the JSON line (and surfaces) here")
+    p.add_argument("--out", default=None, help="also write the whole record (and surfaces) here")
     p.add_argument("--clock-log", default=None,
                    help="CSV file for the nvidia-smi clock samples of the timed region (default: a temp file)")
     p.add_argument("--shape", type=int, nargs=3, default=None, metavar=("M", "N", "K"),
@@ -311,6 +314,41 @@ def merge_t0_shards(local, header, dist, device=None, unmeasured=1 << 60, other=
     if np.any((count != 1) & ~pruned):
         raise RuntimeError("sharded sweep: some entries were measured on no rank or on several")
     return np.where(pruned, unmeasured, np.where(measured, stack, 0).sum(axis=0)).astype(np.int64)
+
+
+# The whole record is tens of kilobytes; a reader of the line may take no more than a few.
+LINE_BYTES = 4000
+_LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+              "vs_baseline", "dtype", "data", "config", "gpu_launches", "sm_count", "setup_s", "roughness_cut_pct",
+              "mean_gain_pct", "roofline_all_gemms", "peak_cell", "clocks")
+_LINE_PARTS = {
+    "plain": ("mean_tflops", "p50_tflops", "p99_tflops", "R_N_slice", "R_3D", "roofline_mean_frac"),
+    "smoothed": ("mean_tflops", "p50_tflops", "p99_tflops", "R_N_slice", "R_3D", "roofline_mean_frac"),
+    "roofline": ("bound", "achieved", "peak", "unit", "frac", "mean_frac", "kernel", "traffic", "traffic_cell"),
+    "roofline_capture": ("kernel", "shape", "achieved", "frac", "traffic", "algorithmic_bytes"),
+    "cpu_baseline": ("value", "unit", "cores", "kind", "cpu_model", "blas"),
+    "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "api"),
+}
+
+
+def short_line(record):
+    """What the printed line holds of the whole record: its contract's keys and the results that name the run, numbers
+    within the parts to six digits."""
+    def rounded(x):
+        if isinstance(x, float):
+            return float(f"{x:.6g}")
+        if isinstance(x, dict):
+            return {k: rounded(v) for k, v in x.items()}
+        return [rounded(v) for v in x] if isinstance(x, (list, tuple)) else x
+    line = {k: record[k] for k in _LINE_KEYS if k in record}
+    for part, keys in _LINE_PARTS.items():
+        if part in record:
+            line[part] = {k: rounded(record[part][k]) for k in keys if record[part].get(k) is not None}
+    blas = line.get("cpu_baseline", {}).get("blas")
+    if isinstance(blas, dict):
+        line["cpu_baseline"]["blas"] = " ".join(str(blas[k]) for k in ("name", "version") if k in blas)
+    line["whole_record"] = "one JSON line on standard error; --out"
+    return line
 
 
 def stats_of(rg, grid, t_ns):
@@ -690,8 +728,8 @@ def main():
         "data": "synthetic",
         "config": {"workload": f"BF16 NN GEMM landscape, (M,N,K) in {{128..{Mx} step 128}}^3 = {ncell} cells, "
                                f"U[-1,1) BF16 operands (seed 0), FP32 accumulate/output",
-                   "smoothed": f"best-of-{rg.RG_NUM_VARIANTS} autotune (the paper's 6 tiles and 128x192, each x "
-                               "{split-K 1/2/4/8, stream-K}; 2 cta_group::2 tiles x {split-K 1/2/4/8, stream-K}) + "
+                   "smoothed": f"best-of-{rg.RG_NUM_VARIANTS} autotune (the paper's 6 tiles, 128x192 and 256x192, each "
+                               "x {split-K 1/2/4/8, stream-K}; 3 cta_group::2 tiles x {split-K 1/2/4/8, stream-K}) + "
                                "DP pad/split plan, O(1) lookup",
                    "plain": "fixed 128x128 tile, split 1",
                    "timing": "per cell: 1 warm-up launch, device spin, mean of 5 back-to-back launches between "
@@ -741,7 +779,8 @@ def main():
     rg.rg_plan_free(plan_smooth)
     rg.rg_destroy(ctx)
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(short_line(line)), flush=True)
         if args.out:
             with open(args.out, "w") as f:
                 json.dump(line, f, indent=1)
